@@ -252,34 +252,7 @@ void *kernel_ptr(bool walls, bool pres, bool staged, bool padded)
 
 namespace {
 lbm_status aa_natural(lbm_ctx *ctx);
-size_t state_bytes(const lbm_ctx *ctx)
-{
-    return (size_t)9 * ctx->pitch * ctx->grid.ny * (ctx->grid.precision == 64 ? 8 : 4);
-}
 }  // namespace
-
-cudaError_t lbm_ctx_copy_state(lbm_ctx *ctx, void *dst)
-{
-    if (aa_natural(ctx) != LBM_OK) return cudaErrorLaunchFailure;
-    return cudaMemcpyAsync(dst, ctx->ws + (ctx->cur ? ctx->L.f1 : ctx->L.f0), state_bytes(ctx),
-                           cudaMemcpyDeviceToDevice, ctx->stream);
-}
-
-const void *lbm_ctx_state(const lbm_ctx *ctx)
-{
-    if (aa_natural(const_cast<lbm_ctx *>(ctx)) != LBM_OK) return nullptr;
-    return ctx->ws + (ctx->cur ? ctx->L.f1 : ctx->L.f0);
-}
-
-cudaError_t lbm_ctx_load_state(lbm_ctx *ctx, const void *src)
-{
-    const size_t bytes = state_bytes(ctx);
-    cudaError_t e = cudaMemcpyAsync(ctx->ws + ctx->L.f0, src, bytes, cudaMemcpyDeviceToDevice, ctx->stream);
-    if (e == cudaSuccess && !ctx->inplace)
-        e = cudaMemcpyAsync(ctx->ws + ctx->L.f1, src, bytes, cudaMemcpyDeviceToDevice, ctx->stream);
-    ctx->aa_odd = false;
-    return e;
-}
 
 void *lbm_step_kernel_ptr(int precision, int mode, bool walls, bool pres, bool staged, bool padded)
 {
@@ -465,8 +438,9 @@ lbm_status plan_launch(lbm_ctx *ctx)
     return LBM_OK;
 }
 
+// src_map: tensor map of A.fin where that is not the context's current buffer
 template <typename real, int MODE>
-cudaError_t launch(lbm_ctx *ctx, const lbm::KArgs<real> &A)
+cudaError_t launch(lbm_ctx *ctx, const lbm::KArgs<real> &A, const CUtensorMap *src_map = nullptr)
 {
     void *fn = step_kernel_ptr(ctx, MODE);
     if (MODE == lbm::MODE_STEP && ctx->tile) {
@@ -500,7 +474,7 @@ cudaError_t launch(lbm_ctx *ctx, const lbm::KArgs<real> &A)
             B.poll_limit = 4096;
             fn = (void *)lbm::step_kernel_rows2<true, true, false, true>;
         }
-        const CUtensorMap *m = B.tma ? &ctx->tmap[ctx->cur] : &unused;
+        const CUtensorMap *m = !B.tma ? &unused : (src_map ? src_map : &ctx->tmap[ctx->cur]);
         void *args[] = {(void *)&B, (void *)m};
         if (ctx->pdl && ctx->early && !ctx->fault_skip) {
             // programmatic dependent launch: the kernel waits for the previous
@@ -700,6 +674,28 @@ bool lbm_encode_population_map(CUtensorMap *map, void *base, int pitch, int ny)
 {
     return encode_population_map(map, base, pitch, ny);
 }
+
+namespace {
+template <typename real>
+cudaError_t step_between(lbm_ctx *ctx, const void *fin, void *fout)
+{
+    lbm::KArgs<real> A = make_args<real>(ctx);
+    A.fin = (const real *)fin;
+    A.fout = (real *)fout;
+    CUtensorMap map;
+    if (ctx->tma_ok && !encode_population_map(&map, const_cast<void *>(fin), ctx->pitch, ctx->grid.ny))
+        return cudaErrorInvalidValue;
+    return launch<real, lbm::MODE_STEP>(ctx, A, &map);
+}
+}  // namespace
+
+cudaError_t lbm_ctx_step_between(lbm_ctx *ctx, const void *fin, void *fout)
+{
+    if (ctx->inplace || ctx->mask || ctx->tile) return cudaErrorNotSupported;
+    return ctx->grid.precision == 64 ? step_between<double>(ctx, fin, fout) : step_between<float>(ctx, fin, fout);
+}
+
+int *lbm_ctx_error_word(lbm_ctx *ctx) { return (int *)(ctx->ws + ctx->L.err); }
 
 namespace {
 

@@ -75,19 +75,19 @@ inline int strip_width(int nx, int w_max, bool bc_x)
 
 } // namespace lbm
 
-// The current population state of a context in its own layout (rows of nine
-// planes, plane pitch pitch_of(nx), 9 * pitch * ny values): an asynchronous
-// device copy out of it / into both of its buffers, on the context's stream
-// and without synchronising (the public lbm_populations / lbm_load_populations
-// convert to the plane-major ABI layout and synchronise). lbm_api.cu.
 #ifdef __CUDACC__
 // 2-D tensor map of one FP32 population array (pitch wide, 9 * ny plane-rows)
 // in the form the row-pair stage loads it (lbm_api.cu); false if the driver
 // entry point is unavailable or the layout does not qualify.
 bool lbm_encode_population_map(CUtensorMap *map, void *base, int pitch, int ny);
-cudaError_t lbm_ctx_copy_state(lbm_ctx *ctx, void *dst);
-const void *lbm_ctx_state(const lbm_ctx *ctx);  // the current state buffer itself (device)
-cudaError_t lbm_ctx_load_state(lbm_ctx *ctx, const void *src);
+// One step of a context between two states outside it, each in the context's
+// own layout (rows of nine planes, plane pitch pitch_of(nx), 9 * pitch * ny
+// values, 256-byte aligned), on the context's stream; slots that no population
+// reaches keep their contents in `fout`. The context's own state and step
+// counter are untouched; bad densities are flagged in its error word (device),
+// lbm_ctx_error_word. Two-array contexts without a wall mask. lbm_api.cu.
+cudaError_t lbm_ctx_step_between(lbm_ctx *ctx, const void *fin, void *fout);
+int *lbm_ctx_error_word(lbm_ctx *ctx);
 
 namespace lbm {
 template <typename real>
