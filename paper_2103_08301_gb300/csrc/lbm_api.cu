@@ -149,6 +149,8 @@ struct lbm_ctx {
     bool tile_maps_ok = false;  // tmap_tile[] encoded
     CUtensorMap tmap_tile[2];   // the same views with the tile kernel's boxes (T_BOX x 9)
     bool allow_tile = false;    // LBM_OPT_TILE (measured slower than the row-pair kernel)
+    bool t64 = false;           // FP64: the tile kernel (lbm_tile64.cu) for the step and the fields
+    lbm::Tile64 t64p{};
     bool tile = false;          // the plan steps with step_kernel_tile (ntx tiles along x)
     int ntx = 0;
     // fields scratch (allocated on first host-pointer lbm_fields)
@@ -342,6 +344,7 @@ bool encode_population_map(CUtensorMap *map, void *base, int pitch, int ny, int 
 
 int threads_of(const lbm_ctx *ctx, int mode)
 {
+    if (ctx->t64) return ctx->t64p.threads;
     if (mode == lbm::MODE_STEP && ctx->rows2) return lbm::R2_BLOCK;
     return cta_threads(ctx->grid.precision, ctx->staged);
 }
@@ -412,6 +415,18 @@ lbm_status plan_launch(lbm_ctx *ctx)
                                              (int)dyn_smem(ctx, lbm::MODE_STEP));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "smem attribute");
     }
+    // FP64: tiles (4096 x 512: 765 us by strips; see lbm_tile64.cuh). The strip
+    // kernels remain for an explicit strip width and unstaged runs.
+    ctx->t64 = false;
+    if (ctx->grid.precision == 64 && ctx->allow_staged && ctx->W_opt == 0) {
+        cudaError_t e = lbm::tile64_plan(nx, ctx->grid.ny, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->sms, &ctx->t64p);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy");
+        ctx->t64 = true;
+        ctx->nctas = ctx->t64p.ctas;
+        if (ctx->ctas_per_sm_opt > 0)
+            ctx->nctas = (int)std::min<long long>({(long long)ctx->sms * ctx->ctas_per_sm_opt, ctx->t64p.ntiles,
+                                                   lbm::MAX_CTAS});
+    }
     // short segments with tensor-load staging: one CTA per 32 x 8 tile instead
     // (no tile boundary between the wall-shear rows ny-3 | ny-2, and the
     // outlet column never alone in a tile: its stencil reaches two columns back)
@@ -442,6 +457,11 @@ lbm_status plan_launch(lbm_ctx *ctx)
 template <typename real, int MODE>
 cudaError_t launch(lbm_ctx *ctx, const lbm::KArgs<real> &A, const CUtensorMap *src_map = nullptr)
 {
+    if constexpr (sizeof(real) == 8) {
+        if (ctx->t64)
+            return lbm::tile64_launch(A, MODE, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->t64p, ctx->nctas,
+                                      ctx->stream);
+    }
     void *fn = step_kernel_ptr(ctx, MODE);
     if (MODE == lbm::MODE_STEP && ctx->tile) {
         // one CTA per 32 x 8 tile, every stencil row staged by a tensor load
@@ -1375,7 +1395,7 @@ extern "C" lbm_status lbm_step_noalloc(const lbm_grid *grid, const lbm_eos *eos,
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return LBM_ERR_CUDA;
     if (plan_launch(&c) != LBM_OK) return LBM_ERR_CUDA;
-    if (ctas > 0) c.nctas = (int)std::min<long long>(ctas, std::max<long long>(1, c.units / 2));
+    if (ctas > 0) c.nctas = (int)std::min<long long>(ctas, c.t64 ? c.t64p.ntiles : std::max<long long>(1, c.units / 2));
     c.nctas = std::min(c.nctas, NOALLOC_MAX_CTAS);
     c.band = band_rows(c.nyf, c.nstrips, c.nctas, c.grid.walls);
     return grid->precision == 64 ? noalloc_launch<double>(&c, sc, f_in, f_out, diag_out, err_out)

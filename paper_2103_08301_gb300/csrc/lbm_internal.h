@@ -134,3 +134,16 @@ void *lbm_step_kernel_ptr(int precision, int mode, bool walls, bool pres, bool s
 // row-pair step likewise, for grids whose 9 pitch ny slots reach 2^31.
 void *lbm_big_step_kernel_ptr(int precision, int mode, bool walls, bool pres, bool staged, bool padded);
 void *lbm_big_rows2_kernel_ptr(bool walls, bool pres, bool padded);
+
+#ifdef __CUDACC__
+namespace lbm {
+// The FP64 step and fields by tiles (lbm_tile64.cu): tile height, grid and CTA
+// count for a lattice, and one launch over `ctas` CTAs (diagnostic slots).
+struct Tile64 {
+    int th, ntx, ntiles, sx, sy, ctas, threads;
+};
+cudaError_t tile64_plan(int nx, int ny, bool walls, bool pres, bool big, int sms, Tile64 *p);
+cudaError_t tile64_launch(const KArgs<double> &A, int mode, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
+                          cudaStream_t st);
+}  // namespace lbm
+#endif

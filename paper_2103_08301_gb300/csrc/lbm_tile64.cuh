@@ -1,0 +1,296 @@
+// The FP64 step and fields by tiles of 32 columns by th rows, one node per
+// thread.
+//
+// GB300 runs FP64 at 1/64 of the FP32 rate (two thread-instructions per clock
+// and SM), so an FP64 step is bound by each SM's FP64 pipe: what counts is the
+// number of FP64 instructions per node, that the pipe of every SM has work all
+// the time, and that the SMs finish together. The strip kernel
+// (lbm_kernels.cuh) holds 90 KB of stage and rings per CTA: two CTAs of four
+// warps per SM, a barrier per row, 82% of the pipe on busy SMs and SMs busy 90%
+// of the step; and a small grid gives it few CTAs (128 x 128: 64, each a serial
+// chain of seven rows). Here a CTA needs only the densities, phi and Laplacians
+// of its tile (no stage: a node's populations stay in its thread's registers),
+// the tiles are many and independent, and the tile height follows the grid so
+// that the SMs' shares are even. FP64 instructions per node are the strip
+// kernel's within 2% (the tile's halo: densities on (32 + 4)(th + 4) points,
+// phi and Laplacian on (32 + 2)(th + 2)). The node arithmetic is the same helper
+// sequence in the same order, so the kernels give identical results.
+//
+// Phases, a barrier after each: (1) densities and phi; (2) Laplacian; (3) force,
+// collision, boundaries, push, diagnostics. CTAs stride over the tiles.
+#pragma once
+
+namespace lbm {
+
+constexpr int T64_TX = 32, T64_MAX = 8;  // tile columns; most rows
+constexpr int T64_AW = T64_TX + 4, T64_BW = T64_TX + 2;
+
+struct SmemT64 {
+    double rho[T64_AW * (T64_MAX + 4)];
+    double phi[T64_BW * (T64_MAX + 2)];
+    double lap[T64_BW * (T64_MAX + 2)];
+    double wv[T64_TX * T64_MAX];  // v_x of the rows next to the walls
+    double red[T64_MAX][2];
+    double ext[T64_MAX][4];
+    int bad;
+};
+
+// Tile grid: th rows per tile, shifted one column left when the outlet column
+// would open a tile (its stencil is its neighbour's), one row down when no height
+// keeps the two rows next to a wall in one tile.
+struct T64Plan {
+    int th, ntx, ntiles, sx, sy;
+};
+
+// row pointers of a shared array as the 3 x 3 operands of the stencils
+template <int SW>
+__device__ __forceinline__ Row3<double> row3d(const double *a, int r, int c)
+{
+    const double *p = a + r * SW + c;
+    return Row3<double>{p[-1], p[0], p[1]};
+}
+
+template <bool WALLS, bool PRES, int MODE, typename IX>
+__global__ void __launch_bounds__(T64_TX *T64_MAX, 2) step_kernel_tile64(const KArgs<double> A, const T64Plan T)
+{
+    using real = double;
+    __shared__ SmemT64 S;
+    const int tid = threadIdx.x, tx = tid & (T64_TX - 1), ty = tid >> 5, th = T.th, tn = T64_TX * th;
+    const int nx = A.nx, ny = A.ny, P = A.pitch, rstride = 9 * P;
+    const int yf0 = WALLS ? 1 : 0, yf1 = WALLS ? ny - 1 : ny;  // fluid rows yf0 .. yf1-1
+    const real third = real(1.0 / 3.0);
+    const Geom<real> G{A.fin, A.fout, nx, ny, A.W, P, A.rho_in_g, A.rho_in_l, A.rho_out_g, A.rho_out_l};
+    Acc<real, 1> acc;
+    acc.reset();
+
+    // density and (want) phi of a stencil point (x, y) up to two nodes off the
+    // lattice; a pressure column's density comes from its interior neighbour
+    auto sum_at = [&](const real *p) {
+        const real s = add_(add_(add_(p[0], p[P]), add_(p[2 * P], p[3 * P])),
+                            add_(add_(p[4 * P], p[5 * P]), add_(p[6 * P], p[7 * P])));
+        return add_(s, p[8 * P]);
+    };
+    auto column_of = [&](int x) {
+        if (PRES) return min(max(x, 1), nx - 2);
+        const int r = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+        return r >= 0 && r < nx ? r : ((x % nx) + nx) % nx;
+    };
+    const int cta = A.reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+
+    for (int t = cta; t < T.ntiles; t += gridDim.x) {
+        const int by = t / T.ntx;
+        const int x0 = (t - by * T.ntx) * T64_TX - T.sx, y0 = yf0 + by * th - T.sy;
+        const int xa = x0 + tx, r = y0 + ty;
+        const bool active = xa >= 0 && xa < nx && r >= yf0 && r < yf1;
+        const bool pin = PRES && active && xa == 0, pout = PRES && active && xa == nx - 1;
+        const bool anyp = pin || pout;
+
+        // (1) densities, phi. Points beyond what the tile's nodes reach read a
+        // clamped node's populations (finite, unused).
+        auto density = [&](int c, int q) {  // local column -2 .. 33, row -2 .. th+1
+            const int x = x0 + c, y = min(y0 + q, yf1 + 1);
+            bool mir;
+            const int row = map_row<WALLS>(y, ny, mir);
+            real s = sum_at(G.fin + (IX)row * rstride + column_of(x));
+            if (PRES && (x <= 0 || x >= nx - 1)) s = column_density(A, G, x >= nx - 1, s);
+            return add_(s, mir ? A.wet : real(0));
+        };
+        real f[9];
+        {
+            const int row = min(max(r, yf0), yf1 - 1);
+            const real *p = G.fin + (IX)row * rstride + column_of(xa);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = __ldg(p + i * P);
+        }
+        for (int h = tid; h < T64_AW * (th + 4) - tn; h += tn) {
+            int c, q;
+            if (h < 4 * T64_AW) {
+                const int k = h / T64_AW;
+                c = h - k * T64_AW - 2;
+                q = k < 2 ? k - 2 : th + k - 2;
+            } else {
+                const int k = (h - 4 * T64_AW) & 3;
+                q = (h - 4 * T64_AW) >> 2;
+                c = k < 2 ? k - 2 : T64_TX + k - 2;
+            }
+            const real v = density(c, q);
+            S.rho[(q + 2) * T64_AW + c + 2] = v;
+            if (c >= -1 && c <= T64_TX && q >= -1 && q <= th) S.phi[(q + 1) * T64_BW + c + 1] = eos_phi<real>(A, v);
+        }
+        {
+            real s = add_(add_(add_(f[0], f[1]), add_(f[2], f[3])), add_(add_(f[4], f[5]), add_(f[6], f[7])));
+            s = add_(s, f[8]);
+            if (PRES && (xa <= 0 || xa >= nx - 1)) s = column_density(A, G, xa >= nx - 1, s);
+            // a tile's rows beyond the fluid are its halo
+            s = r < yf0 || r >= yf1 ? density(tx, ty) : add_(s, real(0));
+            S.rho[(ty + 2) * T64_AW + tx + 2] = s;
+            S.phi[(ty + 1) * T64_BW + tx + 1] = eos_phi<real>(A, s);
+        }
+        __syncthreads();
+
+        // (2) Laplacian on the tile and one node around it
+        auto lap = [&](int c, int q) {
+            S.lap[(q + 1) * T64_BW + c + 1] = lap9<real>(row3d<T64_AW>(S.rho, q + 1, c + 2), row3d<T64_AW>(S.rho, q + 2, c + 2),
+                                                         row3d<T64_AW>(S.rho, q + 3, c + 2));
+        };
+        lap(tx, ty);
+        for (int h = tid; h < T64_BW * (th + 2) - tn; h += tn) {
+            if (h < 2 * T64_BW) {
+                const int k = h / T64_BW;
+                lap(h - k * T64_BW - 1, k ? th : -1);
+            } else {
+                lap(((h - 2 * T64_BW) & 1) ? T64_TX : -1, (h - 2 * T64_BW) >> 1);
+            }
+        }
+        __syncthreads();
+
+        // (3) force, collision, push
+        const int lc = pin ? tx + 1 : (pout ? tx - 1 : tx);  // a pressure column collides its neighbour
+        const int ca = lc + 2, cb = lc + 1, qa = ty + 2, qb = ty + 1;
+        real rho = real(0), vx = real(0);
+        if (active) {
+            real ngpx, ngpy, glx, gly;
+            ngrad12<real>(row3d<T64_BW>(S.phi, qb - 1, cb), row3d<T64_BW>(S.phi, qb, cb), row3d<T64_BW>(S.phi, qb + 1, cb),
+                          ngpx, ngpy);
+            grad12<real>(row3d<T64_BW>(S.lap, qb - 1, cb), row3d<T64_BW>(S.lap, qb, cb), row3d<T64_BW>(S.lap, qb + 1, cb),
+                         glx, gly);
+            rho = S.rho[qa * T64_AW + ca];
+            const real kr = mul_(A.kappa, rho);
+            const real Fx = add_(mulk(fma_(kr, glx, ngpx), 1.0 / 12.0), A.gx);
+            const real Fy = add_(mulk(fma_(kr, gly, ngpy), 1.0 / 12.0), A.gy);
+            const real jx = add_(add_(sub_(f[1], f[3]), sub_(f[5], f[6])), sub_(f[8], f[7]));
+            const real jy = sub_(add_(sub_(f[2], f[4]), add_(f[5], f[6])), add_(f[7], f[8]));
+            const real irho = rcp_(rho);
+            const bool wall_row = WALLS && (r <= 2 || r >= ny - 3);
+            real vy = real(0);
+            if (MODE == MODE_FIELDS || anyp || wall_row) {
+                const real ux = mul_(jx, irho), uy = mul_(jy, irho), hFi = mul_(irho, real(0.5));
+                vx = fma_(hFi, Fx, ux);
+                vy = fma_(hFi, Fy, uy);
+            }
+            const real rho_own = anyp ? S.rho[qa * T64_AW + tx + 2] : rho;
+            if (MODE == MODE_STEP) {
+                real fs[9];
+                if (anyp) {
+                    const real mvx = fma_(real(0.5), Fx, jx), mvy = fma_(real(0.5), Fy, jy);
+                    column_extrapolate<real>(A, rho_own, rho, vx, vy, mvx, mvy, f, fs);
+                } else {
+                    const real mx = fma_(A.ushift, Fx, jx), my = fma_(A.ushift, Fy, jy);
+                    real fe[9];
+                    feq_pairs<real>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
+                    if (A.mrt) {
+                        mrt_relax<real, real>(A, f, fe, fs);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 9; ++i) fs[i] = fma_(sub_(fe[i], f[i]), A.inv_tau, f[i]);
+                    }
+                }
+                real *const out = G.fout;
+                const IX oi = (IX)r * rstride + xa;
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    int x = xa + ex_(i), y = r + ey_(i);
+                    if (WALLS && (y == 0 || y == ny - 1)) {
+                        out[oi + opp_(i) * P] = fs[i];  // half-way bounce-back
+                        continue;
+                    }
+                    if (PRES) {
+                        if (x < 0 || x >= nx) continue;  // leaves through the column
+                    } else {
+                        x = x < 0 ? x + nx : (x >= nx ? x - nx : x);
+                    }
+                    if (!WALLS) y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+                    out[(IX)y * rstride + i * P + x] = fs[i];
+                }
+                acc.mass += rho_own;
+                acc.rmin = vmin_(acc.rmin, rho);
+                acc.rmax = vmax_(acc.rmax, rho);
+            } else {
+                const long long oi = (long long)r * nx + xa;
+                A.o_rho[oi] = rho_own;
+                A.o_vx[oi] = vx;
+                A.o_vy[oi] = vy;
+            }
+            if (WALLS && wall_row) S.wv[tid] = vx;
+        }
+        if (WALLS) {
+            // wall shear: quadratic through v = 0 on the half-way plane and v at
+            // distances 1/2 and 3/2 (both rows lie in this tile); wall pressure:
+            // Eq. 2.4 in mesh units
+            const bool low = y0 <= 1, high = y0 + th >= yf1;  // uniform
+            if (low || high) {
+                __syncthreads();
+                if (active && !anyp) {
+#pragma unroll
+                    for (int side = 0; side < 2; ++side) {
+                        if (r != (side ? ny - 2 : 1)) continue;
+                        const real v2 = S.wv[tid + (side ? -T64_TX : T64_TX)];
+                        const real tw = mul_(mul_(rho, A.nu), mul_(fma_(real(9), vx, -v2), third));
+                        real grx, gry;
+                        grad12<real>(row3d<T64_AW>(S.rho, qa - 1, ca), row3d<T64_AW>(S.rho, qa, ca),
+                                     row3d<T64_AW>(S.rho, qa + 1, ca), grx, gry);
+                        grx = mulk(grx, 1.0 / 12.0);
+                        gry = mulk(gry, 1.0 / 12.0);
+                        const real k2p0 = add_(S.phi[qb * T64_BW + cb], mulk(rho, 1.0 / 3.0));
+                        const real tt = fma_(mul_(A.kappa, rho), -S.lap[qb * T64_BW + cb], k2p0);
+                        const real pw = fma_(fma_(grx, grx, mul_(gry, gry)), mul_(real(-0.5), A.kappa), tt);
+                        if (MODE == MODE_STEP) {
+                            acc.J += tw;
+                            acc.tmin = fmin(acc.tmin, tw); acc.tmax = fmax(acc.tmax, tw);
+                            acc.pmin = fmin(acc.pmin, pw); acc.pmax = fmax(acc.pmax, pw);
+                        } else {
+                            A.o_tw[side * nx + xa] = tw;
+                            A.o_pw[side * nx + xa] = pw;
+                        }
+                    }
+                }
+            }
+        }
+        __syncthreads();  // the shared arrays serve the next tile
+    }
+    if (MODE != MODE_STEP) return;
+
+    // fixed-order reduction: lanes by butterflies, then the warps in order
+    const int lane = tid & 31, warp = tid >> 5;
+    real e[4] = {acc.tmin, acc.tmax, acc.pmin, acc.pmax};
+    const bool anyw = __any_sync(0xffffffffu, e[0] < real(INFINITY) || e[1] > -real(INFINITY) ||
+                                                  e[2] < real(INFINITY) || e[3] > -real(INFINITY) || acc.J != 0.0);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        acc.mass += __shfl_xor_sync(0xffffffffu, acc.mass, o);
+        if (anyw) {
+            acc.J += __shfl_xor_sync(0xffffffffu, acc.J, o);
+            e[0] = fmin(e[0], __shfl_xor_sync(0xffffffffu, e[0], o));
+            e[1] = fmax(e[1], __shfl_xor_sync(0xffffffffu, e[1], o));
+            e[2] = fmin(e[2], __shfl_xor_sync(0xffffffffu, e[2], o));
+            e[3] = fmax(e[3], __shfl_xor_sync(0xffffffffu, e[3], o));
+        }
+    }
+    const bool wbad = __any_sync(0xffffffffu, acc.bad());
+    if (tid == 0) S.bad = 0;
+    __syncthreads();
+    if (lane == 0) {
+        S.red[warp][0] = acc.mass;
+        S.red[warp][1] = acc.J;
+        for (int k = 0; k < 4; ++k) S.ext[warp][k] = e[k];
+        if (wbad) atomicOr(&S.bad, 1);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double m = 0.0, j = 0.0;
+        for (int w = 0; w < th; ++w) {
+            m += S.red[w][0];
+            j += S.red[w][1];
+            e[0] = fmin(e[0], S.ext[w][0]); e[1] = fmax(e[1], S.ext[w][1]);
+            e[2] = fmin(e[2], S.ext[w][2]); e[3] = fmax(e[3], S.ext[w][3]);
+        }
+        A.mass_part[cta] = m;
+        A.J_acc[cta] += j;
+        real *ex = A.ext + 4 * cta;
+        ex[0] = fmin(ex[0], e[0]); ex[1] = fmax(ex[1], e[1]);
+        ex[2] = fmin(ex[2], e[2]); ex[3] = fmax(ex[3], e[3]);
+        if (S.bad) atomicOr(A.err, 1);
+    }
+}
+
+}  // namespace lbm
