@@ -213,6 +213,7 @@ lbm::KArgs<real> make_args(const lbm_ctx *ctx)
     A.rho_out_l = (real)ctx->rho_out_l;
     A.ph_g = (real)ctx->rho_g;
     A.inv_dph = ctx->rho_l > ctx->rho_g ? (real)(1.0 / (ctx->rho_l - ctx->rho_g)) : real(0);
+    lbm::args64(A, ctx->eos.kappa, ctx->eos.k * ctx->eos.k, ctx->eos.R * ctx->T, ctx->eos.a, ctx->tau);
     A.nu = (real)((ctx->tau - 0.5) / 3.0);
     A.eos_kind = ctx->th.kind;
     A.bpr = (real)ctx->th.b;

@@ -208,6 +208,7 @@ lbm::KArgs<real> physics_args(const lbm_batch *b)
     A.inv_tau = (real)(1.0 / b->tau);
     A.omb = (real)(1.0 - 1.0 / b->tau);
     A.wet = (real)b->wet;
+    lbm::args64(A, b->eos.kappa, b->eos.k * b->eos.k, b->eos.R * b->T, b->eos.a, b->tau);
     A.nu = (real)((b->tau - 0.5) / 3.0);
     A.eos_kind = b->th.kind;
     A.bpr = (real)b->th.b;

@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(AA_THREADS, LBM_AA_MIN_BLOCKS)
         // (2) Laplacian at ring rows 1 .. AA_ROWS-2, columns 1 .. AA_SW-2
         for (int k = tid; k < (AA_ROWS - 2) * (AA_SW - 2); k += AA_THREADS) {
             const int j = 1 + k / (AA_SW - 2), c = 1 + k % (AA_SW - 2);
-            S.lap[j][c] = lap9<real>(row3<real, 1, AA_SW>(S.rho, j - 1, c), row3<real, 1, AA_SW>(S.rho, j, c),
+            S.lap[j][c] = lap_stored<real>(row3<real, 1, AA_SW>(S.rho, j - 1, c), row3<real, 1, AA_SW>(S.rho, j, c),
                                      row3<real, 1, AA_SW>(S.rho, j + 1, c));
         }
         __syncthreads();
@@ -294,15 +294,11 @@ __global__ void __launch_bounds__(AA_THREADS, LBM_AA_MIN_BLOCKS)
         real rho = real(0), vx = real(0);
         if (active) {
             const real (&f)[9] = fcur;
-            real ngpx, ngpy, glx, gly;
-            ngrad12<real>(row3<real, 1, AA_SW>(S.phi, qm, ccol), row3<real, 1, AA_SW>(S.phi, q0, ccol),
-                          row3<real, 1, AA_SW>(S.phi, qp, ccol), ngpx, ngpy);
-            grad12<real>(row3<real, 1, AA_SW>(S.lap, qm, ccol), row3<real, 1, AA_SW>(S.lap, q0, ccol),
-                         row3<real, 1, AA_SW>(S.lap, qp, ccol), glx, gly);
             rho = S.rho[q0][ccol];
-            const real kr = mul_(A.kappa, rho);
-            const real Fx = add_(mulk(fma_(kr, glx, ngpx), 1.0 / 12.0), A.gx);
-            const real Fy = add_(mulk(fma_(kr, gly, ngpy), 1.0 / 12.0), A.gy);
+            real Fx, Fy;
+            node_force(A, rho, row3<real, 1, AA_SW>(S.phi, qm, ccol), row3<real, 1, AA_SW>(S.phi, q0, ccol),
+                    row3<real, 1, AA_SW>(S.phi, qp, ccol), row3<real, 1, AA_SW>(S.lap, qm, ccol),
+                    row3<real, 1, AA_SW>(S.lap, q0, ccol), row3<real, 1, AA_SW>(S.lap, qp, ccol), Fx, Fy);
             const real jx = add_(add_(sub_(f[1], f[3]), sub_(f[5], f[6])), sub_(f[8], f[7]));
             const real jy = sub_(add_(sub_(f[2], f[4]), add_(f[5], f[6])), add_(f[7], f[8]));
             const real irho = rcp_(rho);
@@ -316,13 +312,12 @@ __global__ void __launch_bounds__(AA_THREADS, LBM_AA_MIN_BLOCKS)
             {
                 // shifted equilibrium: momentum j + ushift F, velocity (j + ushift F) / rho
                 const real mx = fma_(A.ushift, Fx, jx), my = fma_(A.ushift, Fy, jy);
-                real fe[9];
-                feq_pairs<real>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
                 if (A.mrt) {
+                    real fe[9];
+                    feq_pairs<real>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
                     mrt_relax<real, real>(A, f, fe, fs);
                 } else {
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) fs[i] = fma_(sub_(fe[i], f[i]), A.inv_tau, f[i]);
+                    node_bgk(A, rho, irho, mx, my, f, fs);
                 }
             }
             if (anyp) {
@@ -354,8 +349,7 @@ __global__ void __launch_bounds__(AA_THREADS, LBM_AA_MIN_BLOCKS)
                 }
             }
             acc.macc = add_(acc.macc, rho_own);
-            acc.rmin = vmin_(acc.rmin, rho);
-            acc.rmax = vmax_(acc.rmax, rho);
+            acc.range(rho);
             if (WALLS && !anyp) {
                 if (y == 1) { S.brho1[lane] = rho; S.bv1[lane] = vx; }
                 if (y == ny - 3) S.tv2[lane] = vx;

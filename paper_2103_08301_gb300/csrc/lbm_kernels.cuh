@@ -81,7 +81,22 @@ struct KArgs {
     real *ext;          // [nctas][4] running tw_min, tw_max, pw_min, pw_max
     int *err;           // nonzero once a bad density was met
     real *o_rho, *o_vx, *o_vy, *o_tw, *o_pw;  // MODE_FIELDS outputs (device)
+    // FP64 only: products of the constants above (args64)
+    real kappa6, k2RT, k2a, it3, it9, it12, it36;
 };
+
+// kappa / 6, k^2 RT, k^2 a and the weights 1/3, 1/9, 1/12, 1/36 over tau
+template <typename real>
+inline void args64(KArgs<real> &A, double kappa, double k2, double RT, double a, double tau)
+{
+    A.kappa6 = (real)(kappa / 6.0);
+    A.k2RT = (real)(k2 * RT);
+    A.k2a = (real)(k2 * a);
+    A.it3 = (real)(1.0 / (3.0 * tau));
+    A.it9 = (real)(1.0 / (9.0 * tau));
+    A.it12 = (real)(1.0 / (12.0 * tau));
+    A.it36 = (real)(1.0 / (36.0 * tau));
+}
 
 // D2Q9 velocities, folded at compile time inside unrolled loops.
 __device__ __forceinline__ constexpr int ex_(int i)
@@ -264,6 +279,12 @@ __device__ __forceinline__ V eos_phi(const KArgs<real> &A, V rho)
     const V om = fma_(eta, bc<V>(-1.0), one);          // 1 - eta
     const V num = fma_(eta, fma_(eta, om, one), one);  // 1 + eta (1 + eta (1 - eta))
     const V ir = rcp_(mul_(mul_(om, om), om));
+    if constexpr (sizeof(real) == 8) {
+        // phi = rho k^2 RT num / (1 - eta)^3 - rho (1/3 + k^2 a rho), four
+        // instructions fewer (FP64 steps are bound by their number)
+        const V t = fma_(rho, -A.k2a, bc<V>(-1.0 / 3.0));
+        return fma_(mul_(mul_(rho, A.k2RT), num), ir, mul_(rho, t));
+    }
     const V p0 = fma_(mul_(rho, rho), bcr<V>(-A.a), mul_(mul_(mul_(rho, bcr<V>(A.RT)), num), ir));
     return sub_(mul_(bcr<V>(A.k2), p0), mulk(rho, 1.0 / 3.0));
 }
@@ -498,6 +519,87 @@ __device__ __forceinline__ V lap9(const Row3<V> &m, const Row3<V> &z, const Row3
     return mulk(fma_(z.c, bc<V>(-20.0), fma_(edges, bc<V>(4.0), corners)), 1.0 / 6.0);
 }
 
+// The stored Laplacian: lap psi, in FP64 6 lap psi (the force takes kappa / 6;
+// one instruction fewer per stencil point).
+template <typename V>
+__device__ __forceinline__ V lap_stored(const Row3<V> &m, const Row3<V> &z, const Row3<V> &p)
+{
+    if constexpr (sizeof(el(m.w, 0)) == 8) {
+        const V edges = add_(add_(z.w, z.e), add_(m.c, p.c));
+        const V corners = add_(add_(m.w, m.e), add_(p.w, p.e));
+        return fma_(z.c, bc<V>(-20.0), fma_(edges, bc<V>(4.0), corners));
+    } else {
+        return lap9<V>(m, z, p);
+    }
+}
+template <typename V>
+__device__ __forceinline__ V lap_of_stored(V lap)
+{
+    if constexpr (sizeof(el(lap, 0)) == 8) return mul_(lap, bc<V>(1.0 / 6.0));
+    else return lap;
+}
+
+// FP64 force F = -grad phi + kappa rho grad lap + G from the rows of phi and of the
+// stored Laplacian: both components of a gradient share the differences along
+// the diagonals, and the scale and G enter by one instruction (25 instead of 29).
+// (FP32: the channel kernels' sequence.)
+__device__ __forceinline__ void node_force(const KArgs<float> &A, float rho, const Row3<float> &pm,
+                                           const Row3<float> &pz, const Row3<float> &pp, const Row3<float> &lm,
+                                           const Row3<float> &lz, const Row3<float> &lp, float &Fx, float &Fy)
+{
+    float ngpx, ngpy, glx, gly;
+    ngrad12<float>(pm, pz, pp, ngpx, ngpy);
+    grad12<float>(lm, lz, lp, glx, gly);
+    const float kr = mul_(A.kappa, rho);
+    Fx = add_(mulk(fma_(kr, glx, ngpx), 1.0 / 12.0), A.gx);
+    Fy = add_(mulk(fma_(kr, gly, ngpy), 1.0 / 12.0), A.gy);
+}
+__device__ __forceinline__ void node_force(const KArgs<double> &A, double rho, const Row3<double> &pm,
+                                           const Row3<double> &pz, const Row3<double> &pp, const Row3<double> &lm,
+                                           const Row3<double> &lz, const Row3<double> &lp, double &Fx, double &Fy)
+{
+    const double pa = sub_(pm.w, pp.e), pb = sub_(pm.e, pp.w);  // minus the differences along (1,1), (-1,1)
+    const double la = sub_(lp.e, lm.w), lb = sub_(lp.w, lm.e);
+    const double ngx = fma_(sub_(pz.w, pz.e), 4.0, sub_(pa, pb)), ngy = fma_(sub_(pm.c, pp.c), 4.0, add_(pa, pb));
+    const double glx = fma_(sub_(lz.e, lz.w), 4.0, sub_(la, lb)), gly = fma_(sub_(lp.c, lm.c), 4.0, add_(la, lb));
+    const double kr = mul_(A.kappa6, rho);
+    Fx = fma_(fma_(kr, glx, ngx), 1.0 / 12.0, A.gx);
+    Fy = fma_(fma_(kr, gly, ngy), 1.0 / 12.0, A.gy);
+}
+
+// FP64 BGK: f* = (1 - 1/tau) f + f_eq / tau with f_eq of feq_pairs; 1/tau sits in
+// the weights, the odd parts enter by multiply-add, 4.5 in the velocities, and
+// tau = 1 (uniform) leaves nothing of f: 32 instructions (41 at tau != 1) for 55.
+// (FP32: f_eq, then f + (f_eq - f) / tau.)
+__device__ __forceinline__ void node_bgk(const KArgs<float> &A, float rho, float irho, float mx, float my,
+                                         const float (&f)[9], float (&fs)[9])
+{
+    float fe[9];
+    feq_pairs<float>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) fs[i] = fma_(sub_(fe[i], f[i]), A.inv_tau, f[i]);
+}
+__device__ __forceinline__ void node_bgk(const KArgs<double> &A, double rho, double irho, double mx, double my,
+                                         const double (&f)[9], double (&fs)[9])
+{
+    const double irs = mul_(irho, 2.1213203435596424);  // sqrt(4.5) / rho
+    const double ux = mul_(mx, irs), uy = mul_(my, irs);
+    const double base = fma_(fma_(ux, ux, mul_(uy, uy)), -1.0 / 3.0, 1.0);
+    const double r1 = mul_(rho, A.it9), r2 = mul_(rho, A.it36);
+    const double s = add_(ux, uy), d = sub_(uy, ux), ms = add_(mx, my), md = sub_(my, mx);
+    const double c1 = mul_(r1, fma_(ux, ux, base)), c2 = mul_(r1, fma_(uy, uy, base));
+    const double c5 = mul_(r2, fma_(s, s, base)), c6 = mul_(r2, fma_(d, d, base));
+    fs[1] = fma_(mx, A.it3, c1); fs[3] = fma_(mx, -A.it3, c1);
+    fs[2] = fma_(my, A.it3, c2); fs[4] = fma_(my, -A.it3, c2);
+    fs[5] = fma_(ms, A.it12, c5); fs[7] = fma_(ms, -A.it12, c5);
+    fs[6] = fma_(md, A.it12, c6); fs[8] = fma_(md, -A.it12, c6);
+    fs[0] = fma_(add_(add_(c1, c2), add_(c5, c6)), -2.0, mul_(rho, A.inv_tau));
+    if (A.omb != 0.0) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fs[i] = fma_(f[i], A.omb, fs[i]);
+    }
+}
+
 // MRT relaxation (Eq. 2.1) f* = f - M^-1 S M (f - f_eq) in the Lallemand-Luo
 // moment basis (rho, e, eps, j_x, q_x, j_y, q_y, p_xx, p_xy): the non-
 // equilibrium moments d = f - f_eq are scaled by s_k / |row_k|^2 and mapped
@@ -567,7 +669,7 @@ __device__ __forceinline__ real wall_pressure(const KArgs<real> &A, const real (
     grx = mulk(grx, 1.0 / 12.0);
     gry = mulk(gry, 1.0 / 12.0);
     const real k2p0 = add_(P[q0][cc], mulk(rho, 1.0 / 3.0));
-    const real t = fma_(mul_(A.kappa, rho), -lap, k2p0);
+    const real t = fma_(mul_(A.kappa, rho), -lap_of_stored<real>(lap), k2p0);
     return fma_(fma_(grx, grx, mul_(gry, gry)), mul_(real(-0.5), A.kappa), t);
 }
 
@@ -581,6 +683,13 @@ __device__ __forceinline__ void two_sum_acc(float &h, float &l, float x)
     h = s;
     l = __fadd_rn(l, err);
 }
+
+__device__ __forceinline__ float vmin_(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ float vmax_(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double vmin_(double a, double b) { return fmin(a, b); }
+__device__ __forceinline__ double vmax_(double a, double b) { return fmax(a, b); }
+__device__ __forceinline__ float2 vmin_(float2 a, float2 b) { return make_float2(fminf(a.x, b.x), fminf(a.y, b.y)); }
+__device__ __forceinline__ float2 vmax_(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
 
 // Per-thread diagnostic accumulators of the states read. The density sum is
 // kept in the working precision and flushed every 16 rows (at most 16 terms
@@ -597,8 +706,21 @@ struct Acc {
     float mhi, mlo;  // FP32 builds: the flushed sums as hi + lo
     V macc, rmin, rmax;
     real tmin, tmax, pmin, pmax;
+    bool off;  // FP64: a density outside (0, 1e30) was met
+    // the density of a node: FP32 keeps its range; FP64 compares its bits, which
+    // order positive doubles, on the integer pipes
+    __device__ __forceinline__ void range(V rho)
+    {
+        if constexpr (PAIR) {
+            rmin = vmin_(rmin, rho);
+            rmax = vmax_(rmax, rho);
+        } else {
+            off = off || (unsigned long long)__double_as_longlong(el(rho, 0)) - 1ull >= 0x46293E5939A08CE9ull;
+        }
+    }
     __device__ __forceinline__ void reset()
     {
+        off = false;
         mass = 0.0; J = 0.0; mhi = mlo = 0.f; macc = bc<V>(0.0);
         rmin = bc<V>(INFINITY); rmax = bc<V>(-INFINITY);
         tmin = pmin = real(INFINITY); tmax = pmax = real(-INFINITY);
@@ -617,19 +739,14 @@ struct Acc {
     // a density that is not in (0, 1e30) or a non-finite mass
     __device__ __forceinline__ bool bad() const
     {
-        bool b = PAIR ? !(mhi - mhi == 0.f) : !(mass - mass == 0.0);
+        bool b = PAIR ? !(mhi - mhi == 0.f) : !(mass - mass == 0.0) || off;
+        if constexpr (PAIR) {
 #pragma unroll
-        for (int k = 0; k < CP; ++k) b = b || !(el(rmin, k) > real(0)) || !(el(rmax, k) < real(1e30));
+            for (int k = 0; k < CP; ++k) b = b || !(el(rmin, k) > real(0)) || !(el(rmax, k) < real(1e30));
+        }
         return b;
     }
 };
-
-__device__ __forceinline__ float vmin_(float a, float b) { return fminf(a, b); }
-__device__ __forceinline__ float vmax_(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double vmin_(double a, double b) { return fmin(a, b); }
-__device__ __forceinline__ double vmax_(double a, double b) { return fmax(a, b); }
-__device__ __forceinline__ float2 vmin_(float2 a, float2 b) { return make_float2(fminf(a.x, b.x), fminf(a.y, b.y)); }
-__device__ __forceinline__ float2 vmax_(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
 
 // Static shared-memory working set of a CTA: the 8-row stencil ring (density,
 // EOS potential, Laplacian; strip plus two halo columns per side) and the
@@ -858,12 +975,12 @@ __device__ __forceinline__ void run_segment(const KArgs<real> &A, const Geom<rea
         if (yy >= ya + 1) {
             const int lr = (yy - 2) & (RING - 1), lm = (yy - 3) & (RING - 1), lp = (yy - 1) & (RING - 1);
             if (active) {
-                const V L = lap9<V>(row3<real, CP, SW>(S.rho, lm, c0 + 2), row3<real, CP, SW>(S.rho, lr, c0 + 2),
+                const V L = lap_stored<V>(row3<real, CP, SW>(S.rho, lm, c0 + 2), row3<real, CP, SW>(S.rho, lr, c0 + 2),
                                     row3<real, CP, SW>(S.rho, lp, c0 + 2));
                 stp<V>(&S.lap[lr][c0 + 2], L);
             }
             if (lhalo >= 0)
-                S.lap[lr][lhalo] = lap9<real>(row3<real, 1, SW>(S.rho, lm, lhalo), row3<real, 1, SW>(S.rho, lr, lhalo),
+                S.lap[lr][lhalo] = lap_stored<real>(row3<real, 1, SW>(S.rho, lm, lhalo), row3<real, 1, SW>(S.rho, lr, lhalo),
                                               row3<real, 1, SW>(S.rho, lp, lhalo));
         }
         if constexpr (STAGED) {
@@ -893,15 +1010,22 @@ __device__ __forceinline__ void run_segment(const KArgs<real> &A, const Geom<rea
                 for (int i = 0; i < 9; ++i) f[i] = ldp<V>(sp + i * SP);
             }
             const int q0 = r & (RING - 1), qm = (r - 1) & (RING - 1), qp = (r + 1) & (RING - 1);
-            V ngpx, ngpy, glx, gly;
-            ngrad12<V>(row3<real, CP, SW>(S.phi, qm, ccol), row3<real, CP, SW>(S.phi, q0, ccol),
-                       row3<real, CP, SW>(S.phi, qp, ccol), ngpx, ngpy);
-            grad12<V>(row3<real, CP, SW>(S.lap, qm, ccol), row3<real, CP, SW>(S.lap, q0, ccol),
-                      row3<real, CP, SW>(S.lap, qp, ccol), glx, gly);
+            V Fx, Fy;
             const V rho = ldp<V>(&S.rho[q0][ccol]);
-            const V kr = mul_(bcr<V>(A.kappa), rho);
-            const V Fx = add_(mulk(fma_(kr, glx, ngpx), 1.0 / 12.0), bcr<V>(A.gx));
-            const V Fy = add_(mulk(fma_(kr, gly, ngpy), 1.0 / 12.0), bcr<V>(A.gy));
+            if constexpr (sizeof(real) == 8) {
+                node_force(A, rho, row3<real, CP, SW>(S.phi, qm, ccol), row3<real, CP, SW>(S.phi, q0, ccol),
+                        row3<real, CP, SW>(S.phi, qp, ccol), row3<real, CP, SW>(S.lap, qm, ccol),
+                        row3<real, CP, SW>(S.lap, q0, ccol), row3<real, CP, SW>(S.lap, qp, ccol), Fx, Fy);
+            } else {
+                V ngpx, ngpy, glx, gly;
+                ngrad12<V>(row3<real, CP, SW>(S.phi, qm, ccol), row3<real, CP, SW>(S.phi, q0, ccol),
+                           row3<real, CP, SW>(S.phi, qp, ccol), ngpx, ngpy);
+                grad12<V>(row3<real, CP, SW>(S.lap, qm, ccol), row3<real, CP, SW>(S.lap, q0, ccol),
+                          row3<real, CP, SW>(S.lap, qp, ccol), glx, gly);
+                const V kr = mul_(bcr<V>(A.kappa), rho);
+                Fx = add_(mulk(fma_(kr, glx, ngpx), 1.0 / 12.0), bcr<V>(A.gx));
+                Fy = add_(mulk(fma_(kr, gly, ngpy), 1.0 / 12.0), bcr<V>(A.gy));
+            }
             const V jx = add_(add_(sub_(f[1], f[3]), sub_(f[5], f[6])), sub_(f[8], f[7]));
             const V jy = sub_(add_(sub_(f[2], f[4]), add_(f[5], f[6])), add_(f[7], f[8]));
             const V irho = rcp_(rho);
@@ -916,13 +1040,22 @@ __device__ __forceinline__ void run_segment(const KArgs<real> &A, const Geom<rea
                 {
                     // shifted equilibrium: momentum j + ushift F, velocity (j + ushift F) / rho
                     const V mx = fma_(bcr<V>(A.ushift), Fx, jx), my = fma_(bcr<V>(A.ushift), Fy, jy);
-                    V fe[9];
-                    feq_pairs<V>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
-                    if (A.mrt) {
-                        mrt_relax<V, real>(A, f, fe, fs);
-                    } else {
+                    bool done = false;
+                    if constexpr (sizeof(real) == 8) {
+                        if (!A.mrt) {
+                            node_bgk(A, rho, irho, mx, my, f, fs);
+                            done = true;
+                        }
+                    }
+                    if (!done) {
+                        V fe[9];
+                        feq_pairs<V>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
+                        if (A.mrt) {
+                            mrt_relax<V, real>(A, f, fe, fs);
+                        } else {
 #pragma unroll
-                        for (int i = 0; i < 9; ++i) fs[i] = fma_(sub_(fe[i], f[i]), bcr<V>(A.inv_tau), f[i]);
+                            for (int i = 0; i < 9; ++i) fs[i] = fma_(sub_(fe[i], f[i]), bcr<V>(A.inv_tau), f[i]);
+                        }
                     }
                 }
                 if (anyp) {
@@ -993,8 +1126,7 @@ __device__ __forceinline__ void run_segment(const KArgs<real> &A, const Geom<rea
                     }
                 }
                 acc.macc = add_(acc.macc, rho_own);
-                acc.rmin = vmin_(acc.rmin, rho);
-                acc.rmax = vmax_(acc.rmax, rho);
+                acc.range(rho);
             } else {
 #pragma unroll
                 for (int k = 0; k < CP; ++k) {

@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(MB) mask_phi_lap_kernel(const KArgs<real> A, c
         const Row3<real> rm{E[c - m.sx - 1], E[c - m.sx], E[c - m.sx + 1]};
         const Row3<real> rz{E[c - 1], E[c], E[c + 1]};
         const Row3<real> rp{E[c + m.sx - 1], E[c + m.sx], E[c + m.sx + 1]};
-        La[c] = lap9<real>(rm, rz, rp);
+        La[c] = lap_stored<real>(rm, rz, rp);
     }
 }
 
@@ -153,13 +153,10 @@ __global__ void __launch_bounds__(MB) mask_collide_kernel(const KArgs<real> A, c
         const int rs = y * rstride + xs;
 #pragma unroll
         for (int i = 0; i < 9; ++i) f[i] = A.fin[rs + i * P];
-        real ngpx, ngpy, glx, gly;
-        ngrad12<real>(row3e(Pa, c - sx), row3e(Pa, c), row3e(Pa, c + sx), ngpx, ngpy);
-        grad12<real>(row3e(La, c - sx), row3e(La, c), row3e(La, c + sx), glx, gly);
         const real rho = E[c];
-        const real kr = mul_(A.kappa, rho);
-        const real Fx = add_(mulk(fma_(kr, glx, ngpx), 1.0 / 12.0), A.gx);
-        const real Fy = add_(mulk(fma_(kr, gly, ngpy), 1.0 / 12.0), A.gy);
+        real Fx, Fy;
+        node_force(A, rho, row3e(Pa, c - sx), row3e(Pa, c), row3e(Pa, c + sx), row3e(La, c - sx), row3e(La, c),
+                   row3e(La, c + sx), Fx, Fy);
         const real jx = add_(add_(sub_(f[1], f[3]), sub_(f[5], f[6])), sub_(f[8], f[7]));
         const real jy = sub_(add_(sub_(f[2], f[4]), add_(f[5], f[6])), add_(f[7], f[8]));
         const real irho = rcp_(rho);
@@ -178,13 +175,12 @@ __global__ void __launch_bounds__(MB) mask_collide_kernel(const KArgs<real> A, c
                 column_extrapolate<real>(A, rho_own, rho, vx, vy, mvx, mvy, f, fs);
             } else {
                 const real mx = fma_(A.ushift, Fx, jx), my = fma_(A.ushift, Fy, jy);
-                real fe[9];
-                feq_pairs<real>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
                 if (A.mrt) {
+                    real fe[9];
+                    feq_pairs<real>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
                     mrt_relax<real, real>(A, f, fe, fs);
                 } else {
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) fs[i] = fma_(sub_(fe[i], f[i]), A.inv_tau, f[i]);
+                    node_bgk(A, rho, irho, mx, my, f, fs);
                 }
             }
             const int oi = y * rstride + xa;
@@ -219,7 +215,7 @@ __global__ void __launch_bounds__(MB) mask_collide_kernel(const KArgs<real> A, c
                 grx = mulk(grx, 1.0 / 12.0);
                 gry = mulk(gry, 1.0 / 12.0);
                 const real k2p0 = add_(Pa[c], mulk(rho, 1.0 / 3.0));
-                const real t = fma_(mul_(A.kappa, rho), -La[c], k2p0);
+                const real t = fma_(mul_(A.kappa, rho), -lap_of_stored<real>(La[c]), k2p0);
                 const real pwv = fma_(fma_(grx, grx, mul_(gry, gry)), mul_(real(-0.5), A.kappa), t);
                 if (y == 1) pw[xa] = pwv;
                 if (y == ny - 2) pw[nx + xa] = pwv;

@@ -51,7 +51,7 @@ __device__ __forceinline__ Row3<double> row3d(const double *a, int r, int c)
 }
 
 template <bool WALLS, bool PRES, int MODE, typename IX>
-__global__ void __launch_bounds__(T64_TX *T64_MAX, 2) step_kernel_tile64(const KArgs<double> A, const T64Plan T)
+__global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const KArgs<double> A, const T64Plan T)
 {
     using real = double;
     __shared__ SmemT64 S;
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 2) step_kernel_tile64(const K
 
         // (2) Laplacian on the tile and one node around it
         auto lap = [&](int c, int q) {
-            S.lap[(q + 1) * T64_BW + c + 1] = lap9<real>(row3d<T64_AW>(S.rho, q + 1, c + 2), row3d<T64_AW>(S.rho, q + 2, c + 2),
+            S.lap[(q + 1) * T64_BW + c + 1] = lap_stored<real>(row3d<T64_AW>(S.rho, q + 1, c + 2), row3d<T64_AW>(S.rho, q + 2, c + 2),
                                                          row3d<T64_AW>(S.rho, q + 3, c + 2));
         };
         lap(tx, ty);
@@ -149,15 +149,11 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 2) step_kernel_tile64(const K
         const int ca = lc + 2, cb = lc + 1, qa = ty + 2, qb = ty + 1;
         real rho = real(0), vx = real(0);
         if (active) {
-            real ngpx, ngpy, glx, gly;
-            ngrad12<real>(row3d<T64_BW>(S.phi, qb - 1, cb), row3d<T64_BW>(S.phi, qb, cb), row3d<T64_BW>(S.phi, qb + 1, cb),
-                          ngpx, ngpy);
-            grad12<real>(row3d<T64_BW>(S.lap, qb - 1, cb), row3d<T64_BW>(S.lap, qb, cb), row3d<T64_BW>(S.lap, qb + 1, cb),
-                         glx, gly);
             rho = S.rho[qa * T64_AW + ca];
-            const real kr = mul_(A.kappa, rho);
-            const real Fx = add_(mulk(fma_(kr, glx, ngpx), 1.0 / 12.0), A.gx);
-            const real Fy = add_(mulk(fma_(kr, gly, ngpy), 1.0 / 12.0), A.gy);
+            real Fx, Fy;
+            node_force(A, rho, row3d<T64_BW>(S.phi, qb - 1, cb), row3d<T64_BW>(S.phi, qb, cb),
+                       row3d<T64_BW>(S.phi, qb + 1, cb), row3d<T64_BW>(S.lap, qb - 1, cb), row3d<T64_BW>(S.lap, qb, cb),
+                       row3d<T64_BW>(S.lap, qb + 1, cb), Fx, Fy);
             const real jx = add_(add_(sub_(f[1], f[3]), sub_(f[5], f[6])), sub_(f[8], f[7]));
             const real jy = sub_(add_(sub_(f[2], f[4]), add_(f[5], f[6])), add_(f[7], f[8]));
             const real irho = rcp_(rho);
@@ -176,13 +172,12 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 2) step_kernel_tile64(const K
                     column_extrapolate<real>(A, rho_own, rho, vx, vy, mvx, mvy, f, fs);
                 } else {
                     const real mx = fma_(A.ushift, Fx, jx), my = fma_(A.ushift, Fy, jy);
-                    real fe[9];
-                    feq_pairs<real>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
                     if (A.mrt) {
+                        real fe[9];
+                        feq_pairs<real>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
                         mrt_relax<real, real>(A, f, fe, fs);
                     } else {
-#pragma unroll
-                        for (int i = 0; i < 9; ++i) fs[i] = fma_(sub_(fe[i], f[i]), A.inv_tau, f[i]);
+                        node_bgk(A, rho, irho, mx, my, f, fs);
                     }
                 }
                 real *const out = G.fout;
@@ -203,8 +198,7 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 2) step_kernel_tile64(const K
                     out[(IX)y * rstride + i * P + x] = fs[i];
                 }
                 acc.mass += rho_own;
-                acc.rmin = vmin_(acc.rmin, rho);
-                acc.rmax = vmax_(acc.rmax, rho);
+                acc.range(rho);
             } else {
                 const long long oi = (long long)r * nx + xa;
                 A.o_rho[oi] = rho_own;
@@ -232,7 +226,7 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 2) step_kernel_tile64(const K
                         grx = mulk(grx, 1.0 / 12.0);
                         gry = mulk(gry, 1.0 / 12.0);
                         const real k2p0 = add_(S.phi[qb * T64_BW + cb], mulk(rho, 1.0 / 3.0));
-                        const real tt = fma_(mul_(A.kappa, rho), -S.lap[qb * T64_BW + cb], k2p0);
+                        const real tt = fma_(mul_(A.kappa, rho), -lap_of_stored<real>(S.lap[qb * T64_BW + cb]), k2p0);
                         const real pw = fma_(fma_(grx, grx, mul_(gry, gry)), mul_(real(-0.5), A.kappa), tt);
                         if (MODE == MODE_STEP) {
                             acc.J += tw;
