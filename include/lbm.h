@@ -196,8 +196,7 @@ lbm_status lbm_init(const lbm_grid *grid, const lbm_eos *eos, double tau, const 
  * TMA, TILE, STRIP, CTAS_PER_SM, PREFETCH, PDL) affect only lbm_fields.
  * lbm_launch_info reports the step's CTAs, its threads per CTA (FP32: 128,
  * two rows each; FP64: 256), its 32 x 8 tiles as units, and no staging.
- * lbm_fields allocates its output scratch (3 nx ny values plus 4 nx) on first
- * use, as for any context. Errors: as lbm_init. */
+ * Errors: as lbm_init. */
 size_t lbm_workspace_bytes_inplace(const lbm_grid *grid);
 lbm_status lbm_init_inplace(const lbm_grid *grid, const lbm_eos *eos, double tau, double wetting,
                             const lbm_drive *drive, const double *rho0, void *workspace, size_t ws_bytes,
@@ -219,7 +218,10 @@ lbm_status lbm_step(lbm_ctx *ctx, int64_t n);
  *   tau_wall, p_wall: 2*nx values (bottom wall row then top wall row); zero
  *                for pressure columns and channels without walls.
  * Each pointer may be NULL (skipped), a device pointer or a host pointer, of
- * the context precision. Synchronises the stream. */
+ * the context precision. Destinations in the current device's memory, aligned
+ * to their elements, are written by the kernel; the others go through a device
+ * scratch of their size, allocated at the first call that needs it and kept
+ * (with a wall mask also for skipped outputs). Synchronises the stream. */
 lbm_status lbm_fields(lbm_ctx *ctx, void *rho, void *ux, void *uy, void *tau_wall,
                       void *p_wall);
 

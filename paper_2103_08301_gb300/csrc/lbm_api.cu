@@ -155,6 +155,7 @@ struct lbm_ctx {
     int ntx = 0;
     // fields scratch (allocated on first host-pointer lbm_fields)
     unsigned char *fscratch = nullptr;
+    size_t fscratch_bytes = 0;
     // non-blocking NaN check
     int *h_err = nullptr;
     cudaEvent_t err_ev = nullptr;
@@ -233,22 +234,21 @@ lbm::KArgs<real> make_args(const lbm_ctx *ctx)
     return A;
 }
 
-template <typename real, int MODE, bool STAGED, bool PADDED>
+template <typename real, bool STAGED, bool PADDED>
 void *kernel_ptr(bool walls, bool pres)
 {
     using namespace lbm;
-    if (walls && pres) return (void *)step_kernel<real, true, true, MODE, STAGED, PADDED>;
-    if (walls) return (void *)step_kernel<real, true, false, MODE, STAGED, PADDED>;
-    if (pres) return (void *)step_kernel<real, false, true, MODE, STAGED, PADDED>;
-    return (void *)step_kernel<real, false, false, MODE, STAGED, PADDED>;
+    if (walls && pres) return (void *)step_kernel<real, true, true, STAGED, PADDED>;
+    if (walls) return (void *)step_kernel<real, true, false, STAGED, PADDED>;
+    if (pres) return (void *)step_kernel<real, false, true, STAGED, PADDED>;
+    return (void *)step_kernel<real, false, false, STAGED, PADDED>;
 }
 
-template <typename real, int MODE>
+template <typename real>
 void *kernel_ptr(bool walls, bool pres, bool staged, bool padded)
 {
-    if (staged)
-        return padded ? kernel_ptr<real, MODE, true, true>(walls, pres) : kernel_ptr<real, MODE, true, false>(walls, pres);
-    return padded ? kernel_ptr<real, MODE, false, true>(walls, pres) : kernel_ptr<real, MODE, false, false>(walls, pres);
+    if (staged) return padded ? kernel_ptr<real, true, true>(walls, pres) : kernel_ptr<real, true, false>(walls, pres);
+    return padded ? kernel_ptr<real, false, true>(walls, pres) : kernel_ptr<real, false, false>(walls, pres);
 }
 
 }  // namespace
@@ -256,15 +256,6 @@ void *kernel_ptr(bool walls, bool pres, bool staged, bool padded)
 namespace {
 lbm_status aa_natural(lbm_ctx *ctx);
 }  // namespace
-
-void *lbm_step_kernel_ptr(int precision, int mode, bool walls, bool pres, bool staged, bool padded)
-{
-    if (precision == 64)
-        return mode == lbm::MODE_STEP ? kernel_ptr<double, lbm::MODE_STEP>(walls, pres, staged, padded)
-                                      : kernel_ptr<double, lbm::MODE_FIELDS>(walls, pres, staged, padded);
-    return mode == lbm::MODE_STEP ? kernel_ptr<float, lbm::MODE_STEP>(walls, pres, staged, padded)
-                                  : kernel_ptr<float, lbm::MODE_FIELDS>(walls, pres, staged, padded);
-}
 
 namespace {
 
@@ -279,29 +270,28 @@ void *rows2_kernel_ptr(bool walls, bool pres)
 }
 
 
-void *step_kernel_ptr(const lbm_ctx *ctx, int mode)
+void *step_kernel_ptr(const lbm_ctx *ctx)
 {
     const bool padded = ctx->pitch != ctx->grid.nx;
     if (ctx->big) {
-        if (mode == lbm::MODE_STEP && ctx->rows2)
-            return lbm_big_rows2_kernel_ptr(ctx->grid.walls, ctx->grid.bc_x, padded);
-        return lbm_big_step_kernel_ptr(ctx->grid.precision, mode, ctx->grid.walls, ctx->grid.bc_x, ctx->staged,
-                                       padded);
+        if (ctx->rows2) return lbm_big_rows2_kernel_ptr(ctx->grid.walls, ctx->grid.bc_x, padded);
+        return lbm_big_step_kernel_ptr(ctx->grid.precision, ctx->grid.walls, ctx->grid.bc_x, ctx->staged, padded);
     }
-    if (mode == lbm::MODE_STEP && ctx->rows2) {
+    if (ctx->rows2) {
         if (ctx->early)
             return padded ? rows2_kernel_ptr<true, 3>(ctx->grid.walls, ctx->grid.bc_x)
                           : rows2_kernel_ptr<false, 3>(ctx->grid.walls, ctx->grid.bc_x);
         return padded ? rows2_kernel_ptr<true, 1>(ctx->grid.walls, ctx->grid.bc_x)
                       : rows2_kernel_ptr<false, 1>(ctx->grid.walls, ctx->grid.bc_x);
     }
-    return lbm_step_kernel_ptr(ctx->grid.precision, mode, ctx->grid.walls, ctx->grid.bc_x, ctx->staged, padded);
+    return ctx->grid.precision == 64 ? kernel_ptr<double>(ctx->grid.walls, ctx->grid.bc_x, ctx->staged, padded)
+                                     : kernel_ptr<float>(ctx->grid.walls, ctx->grid.bc_x, ctx->staged, padded);
 }
 
-size_t dyn_smem(const lbm_ctx *ctx, int mode)
+size_t dyn_smem(const lbm_ctx *ctx)
 {
     if (!ctx->staged) return 0;
-    if (mode == lbm::MODE_STEP && ctx->rows2) return lbm::rows2_smem_bytes();
+    if (ctx->rows2) return lbm::rows2_smem_bytes();
     return ctx->grid.precision == 64 ? lbm::staged_smem_bytes<double>()
                                      : lbm::staged_smem_bytes<float>();
 }
@@ -343,10 +333,10 @@ bool encode_population_map(CUtensorMap *map, void *base, int pitch, int ny, int 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int threads_of(const lbm_ctx *ctx, int mode)
+int threads_of(const lbm_ctx *ctx)
 {
     if (ctx->t64) return ctx->t64p.threads;
-    if (mode == lbm::MODE_STEP && ctx->rows2) return lbm::R2_BLOCK;
+    if (ctx->rows2) return lbm::R2_BLOCK;
     return cta_threads(ctx->grid.precision, ctx->staged);
 }
 
@@ -388,19 +378,18 @@ lbm_status plan_launch(lbm_ctx *ctx)
     ctx->nyf = ctx->grid.walls ? ctx->grid.ny - 2 : ctx->grid.ny;
     ctx->units = (long long)ctx->nstrips * ctx->nyf;
     ctx->early = false;  // chosen once the CTA count is known
+    ctx->t64 = false;    // likewise
 
-    for (int mode : {lbm::MODE_STEP, lbm::MODE_FIELDS}) {
-        cudaError_t e = cudaFuncSetAttribute(step_kernel_ptr(ctx, mode),
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)dyn_smem(ctx, mode));
+    {
+        cudaError_t e = cudaFuncSetAttribute(step_kernel_ptr(ctx), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)dyn_smem(ctx));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "smem attribute");
     }
     int per_sm = ctx->ctas_per_sm_opt;
     if (per_sm <= 0) {
         int occ = 0;
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &occ, step_kernel_ptr(ctx, lbm::MODE_STEP), threads_of(ctx, lbm::MODE_STEP),
-            dyn_smem(ctx, lbm::MODE_STEP));
+            &occ, step_kernel_ptr(ctx), threads_of(ctx), dyn_smem(ctx));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy");
         per_sm = std::max(1, occ);
     }
@@ -411,14 +400,12 @@ lbm_status plan_launch(lbm_ctx *ctx)
     ctx->band = band_rows(ctx->nyf, ctx->nstrips, ctx->nctas, ctx->grid.walls);
     if (ctx->rows2 && !ctx->big && ctx->units < EARLY_ROWS * ctx->nctas) {
         ctx->early = true;
-        cudaError_t e = cudaFuncSetAttribute(step_kernel_ptr(ctx, lbm::MODE_STEP),
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)dyn_smem(ctx, lbm::MODE_STEP));
+        cudaError_t e = cudaFuncSetAttribute(step_kernel_ptr(ctx), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)dyn_smem(ctx));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "smem attribute");
     }
     // FP64: tiles (4096 x 512: 765 us by strips; see lbm_tile64.cuh). The strip
     // kernels remain for an explicit strip width and unstaged runs.
-    ctx->t64 = false;
     if (ctx->grid.precision == 64 && ctx->allow_staged && ctx->W_opt == 0) {
         cudaError_t e = lbm::tile64_plan(nx, ctx->grid.ny, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->sms, &ctx->t64p);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy");
@@ -455,16 +442,15 @@ lbm_status plan_launch(lbm_ctx *ctx)
 }
 
 // src_map: tensor map of A.fin where that is not the context's current buffer
-template <typename real, int MODE>
+template <typename real>
 cudaError_t launch(lbm_ctx *ctx, const lbm::KArgs<real> &A, const CUtensorMap *src_map = nullptr)
 {
     if constexpr (sizeof(real) == 8) {
         if (ctx->t64)
-            return lbm::tile64_launch(A, MODE, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->t64p, ctx->nctas,
-                                      ctx->stream);
+            return lbm::tile64_launch(A, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->t64p, ctx->nctas, ctx->stream);
     }
-    void *fn = step_kernel_ptr(ctx, MODE);
-    if (MODE == lbm::MODE_STEP && ctx->tile) {
+    void *fn = step_kernel_ptr(ctx);
+    if (ctx->tile) {
         // one CTA per 32 x 8 tile, every stencil row staged by a tensor load
         lbm::KArgs<real> B = A;
         fn = ctx->grid.walls ? (ctx->grid.bc_x ? (void *)lbm::step_kernel_tile<true, true>
@@ -485,7 +471,7 @@ cudaError_t launch(lbm_ctx *ctx, const lbm::KArgs<real> &A, const CUtensorMap *s
         cfg.numAttrs = ctx->pdl ? 1 : 0;
         return cudaLaunchKernelExC(&cfg, fn, args);
     }
-    if (MODE == lbm::MODE_STEP && ctx->rows2) {
+    if (ctx->rows2) {
         // the row-pair kernel also takes the tensor map of its source buffer
         static const CUtensorMap unused{};
         lbm::KArgs<real> B = A;
@@ -507,18 +493,18 @@ cudaError_t launch(lbm_ctx *ctx, const lbm::KArgs<real> &A, const CUtensorMap *s
             at[0].val.programmaticStreamSerializationAllowed = 1;
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(ctx->nctas);
-            cfg.blockDim = dim3(threads_of(ctx, MODE));
-            cfg.dynamicSmemBytes = dyn_smem(ctx, MODE);
+            cfg.blockDim = dim3(threads_of(ctx));
+            cfg.dynamicSmemBytes = dyn_smem(ctx);
             cfg.stream = ctx->stream;
             cfg.attrs = at;
             cfg.numAttrs = 1;
             return cudaLaunchKernelExC(&cfg, fn, args);
         }
-        return cudaLaunchKernel(fn, dim3(ctx->nctas), dim3(threads_of(ctx, MODE)), args, dyn_smem(ctx, MODE),
+        return cudaLaunchKernel(fn, dim3(ctx->nctas), dim3(threads_of(ctx)), args, dyn_smem(ctx),
                                 ctx->stream);
     }
     void *args[] = {(void *)&A};
-    return cudaLaunchKernel(fn, dim3(ctx->nctas), dim3(threads_of(ctx, MODE)), args, dyn_smem(ctx, MODE),
+    return cudaLaunchKernel(fn, dim3(ctx->nctas), dim3(threads_of(ctx)), args, dyn_smem(ctx),
                             ctx->stream);
 }
 
@@ -576,7 +562,7 @@ lbm_status one_step(lbm_ctx *ctx)
         return LBM_OK;
     }
     cudaError_t e = ctx->mask ? lbm::mask_launch<real>(ctx->mask, A, lbm::MODE_STEP, ctx->stream)
-                              : launch<real, lbm::MODE_STEP>(ctx, A);
+                              : launch<real>(ctx, A);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "step launch");
     ctx->cur = 1 - ctx->cur;
     ctx->step += 1;
@@ -628,28 +614,44 @@ template <typename real>
 lbm_status do_fields(lbm_ctx *ctx, void *rho, void *ux, void *uy, void *tw, void *pw)
 {
     if (lbm_status s0 = aa_natural(ctx)) return s0;
-    const size_t N = (size_t)ctx->grid.nx * ctx->grid.ny, nx = ctx->grid.nx;
-    const size_t sz = sizeof(real);
-    if (!ctx->fscratch) {
-        CK(cudaMalloc((void **)&ctx->fscratch, align_up(3 * N * sz) + align_up(4 * nx * sz)),
-           "fields scratch");
+    // device destinations are written by the kernel; others (and, with a wall
+    // mask, absent ones) through a scratch kept from the first call that needs it
+    lbm::FieldsOut<real> o{};
+    void *dst[5] = {rho, ux, uy, tw, pw};
+    for (int k = 0; k < 5; ++k) o.dst[k] = dst[k];
+    lbm::fields_route(o, ctx->grid.nx, ctx->grid.ny, ctx->ws, ctx->L.total);
+    size_t need = o.scratch, spare = 0;
+    if (ctx->mask)
+        for (int k = 0; k < 5; ++k)
+            if (!o.dst[k]) spare += align_up(o.bytes[k]);
+    need += spare;
+    if (need > ctx->fscratch_bytes) {
+        if (ctx->fscratch) cudaFree(ctx->fscratch);
+        ctx->fscratch = nullptr;
+        ctx->fscratch_bytes = 0;
+        CK(cudaMalloc((void **)&ctx->fscratch, need), "fields scratch");
+        ctx->fscratch_bytes = need;
     }
-    real *d_rho = (real *)ctx->fscratch, *d_vx = d_rho + N, *d_vy = d_vx + N;
-    real *d_tw = (real *)(ctx->fscratch + align_up(3 * N * sz)), *d_pw = d_tw + 2 * nx;
-    CK(cudaMemsetAsync(ctx->fscratch, 0, align_up(3 * N * sz) + align_up(4 * nx * sz), ctx->stream),
-       "fields memset");
+    o.use(ctx->fscratch);
     lbm::KArgs<real> A = make_args<real>(ctx);
-    A.fout = nullptr;
-    A.o_rho = d_rho; A.o_vx = d_vx; A.o_vy = d_vy; A.o_tw = d_tw; A.o_pw = d_pw;
-    cudaError_t le = ctx->mask ? lbm::mask_launch<real>(ctx->mask, A, lbm::MODE_FIELDS, ctx->stream)
-                               : launch<real, lbm::MODE_FIELDS>(ctx, A);
-    if (le != cudaSuccess) return cuda_fail(ctx, le, "fields launch");
-    struct { void *dst; real *src; size_t n; } outs[] = {
-        {rho, d_rho, N}, {ux, d_vx, N}, {uy, d_vy, N}, {tw, d_tw, 2 * nx}, {pw, d_pw, 2 * nx}};
-    for (auto &o : outs) {
-        if (!o.dst) continue;
-        CK(cudaMemcpyAsync(o.dst, o.src, o.n * sz, cudaMemcpyDefault, ctx->stream), "fields copy");
+    if (ctx->mask) {
+        A.fout = nullptr;
+        real *p[5];
+        size_t at = o.scratch;
+        for (int k = 0; k < 5; ++k) {
+            p[k] = o.ptr[k];
+            if (!p[k]) {
+                p[k] = (real *)(ctx->fscratch + at);
+                at += align_up(o.bytes[k]);
+            }
+            CK(cudaMemsetAsync(p[k], 0, o.bytes[k], ctx->stream), "fields memset");  // solid nodes
+        }
+        A.o_rho = p[0]; A.o_vx = p[1]; A.o_vy = p[2]; A.o_tw = p[3]; A.o_pw = p[4];
+        CK(lbm::mask_launch<real>(ctx->mask, A, lbm::MODE_FIELDS, ctx->stream), "fields launch");
+    } else {
+        CK(lbm::fields_tiles<real>(A, o, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->sms, ctx->stream), "fields launch");
     }
+    CK(lbm::fields_copy(o, ctx->stream), "fields copy");
     CK(cudaStreamSynchronize(ctx->stream), "fields sync");
     return LBM_OK;
 }
@@ -706,7 +708,7 @@ cudaError_t step_between(lbm_ctx *ctx, const void *fin, void *fout)
     CUtensorMap map;
     if (ctx->tma_ok && !encode_population_map(&map, const_cast<void *>(fin), ctx->pitch, ctx->grid.ny))
         return cudaErrorInvalidValue;
-    return launch<real, lbm::MODE_STEP>(ctx, A, &map);
+    return launch<real>(ctx, A, &map);
 }
 }  // namespace
 
@@ -1245,7 +1247,7 @@ lbm_status lbm_launch_info(const lbm_ctx *ctx, int64_t *ctas, int64_t *threads, 
         return LBM_OK;
     }
     if (ctas) *ctas = ctx->nctas;
-    if (threads) *threads = ctx->mask ? 256 : threads_of(ctx, lbm::MODE_STEP);
+    if (threads) *threads = ctx->mask ? 256 : threads_of(ctx);
     if (units) *units = ctx->mask ? (int64_t)ctx->grid.nx * ctx->grid.ny : ctx->units;
     if (staged) *staged = (ctx->staged && !ctx->mask) ? 1 : 0;
     return LBM_OK;
@@ -1337,7 +1339,7 @@ lbm_status noalloc_launch(lbm_ctx *c, NoallocScratch *sc, const void *f_in, void
     A.J_acc = sc->J;
     A.ext = ext;
     A.err = &sc->err;
-    cudaError_t e = launch<real, lbm::MODE_STEP>(c, A);
+    cudaError_t e = launch<real>(c, A);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "noalloc step");
     if (diag_out)
         lbm::diag_kernel<real><<<1, 256, 0, c->stream>>>(sc->mass, sc->J, ext, &sc->err, c->nctas, diag_out);

@@ -518,51 +518,36 @@ lbm_status upload_chan_table(lbm_batch *b)
     return LBM_OK;
 }
 
-// Macroscopic fields of one channel with the single-channel kernel in fields mode.
+// Macroscopic fields of one channel (the kernel of lbm_fields).
 template <typename real>
 lbm_status chan_fields(lbm_batch *b, int ci, void *rho, void *ux, void *uy, void *tw, void *pw)
 {
     const ChanHost &c = b->ch[ci];
-    const size_t N = (size_t)c.grid.nx * c.grid.ny, nx = c.grid.nx, sz = sizeof(real);
-    const size_t need = (3 * N + 4 * nx) * sz + 256;
-    if (b->fscratch_bytes < need) {
+    lbm::FieldsOut<real> o{};
+    void *dst[5] = {rho, ux, uy, tw, pw};
+    for (int k = 0; k < 5; ++k) o.dst[k] = dst[k];
+    const real *state = reinterpret_cast<const real *>(b->pop[b->cur]) + c.off;
+    lbm::fields_route(o, c.grid.nx, c.grid.ny, state, (size_t)9 * c.pitch * c.grid.ny * sizeof(real));
+    if (b->fscratch_bytes < o.scratch) {
         cudaFree(b->fscratch);
         b->fscratch = nullptr;
-        BCK(cudaMalloc((void **)&b->fscratch, need), "fields scratch");
-        b->fscratch_bytes = need;
+        b->fscratch_bytes = 0;
+        BCK(cudaMalloc((void **)&b->fscratch, o.scratch), "fields scratch");
+        b->fscratch_bytes = o.scratch;
     }
-    real *d_rho = (real *)b->fscratch, *d_vx = d_rho + N, *d_vy = d_vx + N, *d_tw = d_vy + N, *d_pw = d_tw + 2 * nx;
-    BCK(cudaMemsetAsync(b->fscratch, 0, need, b->stream), "fields memset");
+    o.use(b->fscratch);
     lbm::KArgs<real> A = physics_args<real>(b);
-    A.fin = reinterpret_cast<const real *>(b->pop[b->cur]) + c.off;
-    A.fout = nullptr;
-    A.plane = (long long)N;
+    A.fin = state;
+    A.plane = (long long)c.grid.nx * c.grid.ny;
     A.nx = c.grid.nx;
     A.ny = c.grid.ny;
     A.pitch = c.pitch;
-    A.W = c.W;
-    A.nstrips = c.nstrips;
-    A.yf0 = c.yf0;
-    A.nyf = c.nyf;
-    A.units = c.units;
-    A.band = c.nyf;  // strip-major
     A.rho_in_g = (real)c.rho_in;
     A.rho_in_l = (real)c.rho_in_l;
     A.rho_out_g = (real)c.rho_out;
     A.rho_out_l = (real)c.rho_out_l;
-    A.o_rho = d_rho; A.o_vx = d_vx; A.o_vy = d_vy; A.o_tw = d_tw; A.o_pw = d_pw;
-    const bool st = b->allow_staged && c.pitch % 4 == 0 && c.W % 4 == 0;
-    void *fn = lbm_step_kernel_ptr(b->precision, lbm::MODE_FIELDS, b->walls, b->bc_x, st, c.pitch != c.grid.nx);
-    const size_t smem = staged_bytes(b, st);
-    BCK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "smem attribute");
-    A.nctas = (int)std::max<long long>(1, std::min<long long>((long long)b->sms * 4, c.units / 2));
-    void *args[] = {(void *)&A};
-    BCK(cudaLaunchKernel(fn, dim3(A.nctas), dim3(cta_threads(b->precision, st)), args, smem, b->stream),
-        "fields launch");
-    struct { void *dst; real *src; size_t n; } outs[] = {
-        {rho, d_rho, N}, {ux, d_vx, N}, {uy, d_vy, N}, {tw, d_tw, 2 * nx}, {pw, d_pw, 2 * nx}};
-    for (auto &o : outs)
-        if (o.dst) BCK(cudaMemcpyAsync(o.dst, o.src, o.n * sz, cudaMemcpyDefault, b->stream), "fields copy");
+    BCK(lbm::fields_tiles<real>(A, o, b->walls, b->bc_x, false, b->sms, b->stream), "fields launch");
+    BCK(lbm::fields_copy(o, b->stream), "fields copy");
     BCK(cudaStreamSynchronize(b->stream), "fields sync");
     return LBM_OK;
 }

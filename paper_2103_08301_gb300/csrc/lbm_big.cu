@@ -13,22 +13,22 @@ namespace {
 
 using IX = long long;
 
-template <typename real, int MODE, bool STAGED, bool PADDED>
+template <typename real, bool STAGED, bool PADDED>
 void *big_ptr(bool walls, bool pres)
 {
     using namespace lbm;
-    if (walls && pres) return (void *)step_kernel<real, true, true, MODE, STAGED, PADDED, IX>;
-    if (walls) return (void *)step_kernel<real, true, false, MODE, STAGED, PADDED, IX>;
-    if (pres) return (void *)step_kernel<real, false, true, MODE, STAGED, PADDED, IX>;
-    return (void *)step_kernel<real, false, false, MODE, STAGED, PADDED, IX>;
+    if (walls && pres) return (void *)step_kernel<real, true, true, STAGED, PADDED, IX>;
+    if (walls) return (void *)step_kernel<real, true, false, STAGED, PADDED, IX>;
+    if (pres) return (void *)step_kernel<real, false, true, STAGED, PADDED, IX>;
+    return (void *)step_kernel<real, false, false, STAGED, PADDED, IX>;
 }
 
-template <typename real, int MODE>
+template <typename real>
 void *big_ptr(bool walls, bool pres, bool staged, bool padded)
 {
     if (staged)
-        return padded ? big_ptr<real, MODE, true, true>(walls, pres) : big_ptr<real, MODE, true, false>(walls, pres);
-    return padded ? big_ptr<real, MODE, false, true>(walls, pres) : big_ptr<real, MODE, false, false>(walls, pres);
+        return padded ? big_ptr<real, true, true>(walls, pres) : big_ptr<real, true, false>(walls, pres);
+    return padded ? big_ptr<real, false, true>(walls, pres) : big_ptr<real, false, false>(walls, pres);
 }
 
 template <bool PADDED>
@@ -43,13 +43,9 @@ void *big_rows2_ptr(bool walls, bool pres)
 
 } // namespace
 
-void *lbm_big_step_kernel_ptr(int precision, int mode, bool walls, bool pres, bool staged, bool padded)
+void *lbm_big_step_kernel_ptr(int precision, bool walls, bool pres, bool staged, bool padded)
 {
-    if (precision == 64)
-        return mode == lbm::MODE_STEP ? big_ptr<double, lbm::MODE_STEP>(walls, pres, staged, padded)
-                                      : big_ptr<double, lbm::MODE_FIELDS>(walls, pres, staged, padded);
-    return mode == lbm::MODE_STEP ? big_ptr<float, lbm::MODE_STEP>(walls, pres, staged, padded)
-                                  : big_ptr<float, lbm::MODE_FIELDS>(walls, pres, staged, padded);
+    return precision == 64 ? big_ptr<double>(walls, pres, staged, padded) : big_ptr<float>(walls, pres, staged, padded);
 }
 
 void *lbm_big_rows2_kernel_ptr(bool walls, bool pres, bool padded)

@@ -126,13 +126,9 @@ cudaError_t aa_swap(int precision, void *F, bool walls, bool pres, bool big, int
 }  // namespace lbm
 #endif
 
-// Launchable step kernel (lbm_api.cu) for a precision (32/64), a mode
-// (lbm::MODE_STEP or MODE_FIELDS), the boundary set, the staged variant and a
-// row pitch above nx (padded).
-void *lbm_step_kernel_ptr(int precision, int mode, bool walls, bool pres, bool staged, bool padded);
-// The same kernels with 64-bit population offsets (lbm_big.cu), and the FP32
+// The step kernels with 64-bit population offsets (lbm_big.cu), and the FP32
 // row-pair step likewise, for grids whose 9 pitch ny slots reach 2^31.
-void *lbm_big_step_kernel_ptr(int precision, int mode, bool walls, bool pres, bool staged, bool padded);
+void *lbm_big_step_kernel_ptr(int precision, bool walls, bool pres, bool staged, bool padded);
 void *lbm_big_rows2_kernel_ptr(bool walls, bool pres, bool padded);
 
 #ifdef __CUDACC__
@@ -143,7 +139,31 @@ struct Tile64 {
     int th, ntx, ntiles, sx, sy, ctas, threads;
 };
 cudaError_t tile64_plan(int nx, int ny, bool walls, bool pres, bool big, int sms, Tile64 *p);
-cudaError_t tile64_launch(const KArgs<double> &A, int mode, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
+cudaError_t tile64_launch(const KArgs<double> &A, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
                           cudaStream_t st);
+
+// Destinations of the macroscopic fields rho, ux, uy (nx ny values), tau_w, p_w
+// (2 nx), any of them NULL. fields_route decides which a kernel writes itself
+// (device memory of this device that overlaps neither another output nor the
+// `busy` range, the state): ptr = dst; the others need `scratch` bytes, output
+// k at offset[k], which the caller points ptr[k] to. fields_tiles computes the
+// outputs with a ptr; fields_copy brings the scratch ones to their destinations.
+template <typename real>
+struct FieldsOut {
+    void *dst[5];
+    real *ptr[5];
+    size_t bytes[5], offset[5], scratch;
+    void use(unsigned char *mem)
+    {
+        for (int k = 0; k < 5; ++k)
+            if (dst[k] && !ptr[k]) ptr[k] = (real *)(mem + offset[k]);
+    }
+};
+template <typename real>
+void fields_route(FieldsOut<real> &o, int nx, int ny, const void *busy, size_t busy_bytes);
+template <typename real>
+cudaError_t fields_tiles(KArgs<real> A, const FieldsOut<real> &o, bool walls, bool pres, bool big, int sms, cudaStream_t st);
+template <typename real>
+cudaError_t fields_copy(const FieldsOut<real> &o, cudaStream_t st);
 }  // namespace lbm
 #endif

@@ -37,7 +37,7 @@ namespace lbm {
 constexpr int RING = 8;      // shared-memory ring rows (power of two)
 constexpr int MAX_CTAS = 8192;
 
-enum { MODE_STEP = 0, MODE_FIELDS = 1 };
+enum { MODE_STEP = 0, MODE_FIELDS = 1 };  // of the tile and general-geometry kernels
 
 template <typename real>
 struct KArgs {
@@ -761,7 +761,7 @@ struct Smem {
     int bad;
 };
 
-// One fused time step (MODE_STEP) or the macroscopic fields (MODE_FIELDS).
+// One fused time step.
 //
 // Per segment (strip of columns x0 .. x0+xw-1, fluid rows ya .. yb-1) the CTA
 // runs iterations yy = ya-2 .. yb+2 with one barrier each:
@@ -787,8 +787,7 @@ struct Smem {
 // with one row of register prefetch and re-reads the collision row from L1.
 // In both variants four halo lanes load the two columns beyond each strip
 // edge with one row of register prefetch.
-template <typename real, bool WALLS, bool PRES, int MODE, int BLOCK, bool STAGED, int CP, bool PADDED,
-          typename IX = int>
+template <typename real, bool WALLS, bool PRES, int BLOCK, bool STAGED, int CP, bool PADDED, typename IX = int>
 __device__ __forceinline__ void run_segment(const KArgs<real> &A, const Geom<real> &G, int s, int ya, int yb,
                                             Smem<real, BLOCK> &S, real *stages, uint64_t *bars,
                                             RingPos &ring_next, Acc<real, CP> &acc, bool &lost)
@@ -1035,109 +1034,97 @@ __device__ __forceinline__ void run_segment(const KArgs<real> &A, const Geom<rea
             // own-column density (a pressure column's own is rho_b)
             const V rho_own = (CP == 1 && anyp) ? bcr<V>(S.rho[q0][tid + 2]) : rho;
 
-            if (MODE == MODE_STEP) {
-                V fs[9];
-                {
-                    // shifted equilibrium: momentum j + ushift F, velocity (j + ushift F) / rho
-                    const V mx = fma_(bcr<V>(A.ushift), Fx, jx), my = fma_(bcr<V>(A.ushift), Fy, jy);
-                    bool done = false;
-                    if constexpr (sizeof(real) == 8) {
-                        if (!A.mrt) {
-                            node_bgk(A, rho, irho, mx, my, f, fs);
-                            done = true;
-                        }
-                    }
-                    if (!done) {
-                        V fe[9];
-                        feq_pairs<V>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
-                        if (A.mrt) {
-                            mrt_relax<V, real>(A, f, fe, fs);
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 9; ++i) fs[i] = fma_(sub_(fe[i], f[i]), bcr<V>(A.inv_tau), f[i]);
-                        }
+            V fs[9];
+            {
+                // shifted equilibrium: momentum j + ushift F, velocity (j + ushift F) / rho
+                const V mx = fma_(bcr<V>(A.ushift), Fx, jx), my = fma_(bcr<V>(A.ushift), Fy, jy);
+                bool done = false;
+                if constexpr (sizeof(real) == 8) {
+                    if (!A.mrt) {
+                        node_bgk(A, rho, irho, mx, my, f, fs);
+                        done = true;
                     }
                 }
-                if (anyp) {
-                    // pressure column: extrapolate from the interior neighbour
-                    // (CP = 1: this thread's values are the neighbour's; pairs:
-                    // the other element of the pair)
-                    const int kc = pin ? 0 : CP - 1, kf = (CP == 1) ? 0 : (pin ? 1 : CP - 2);
-                    real ff[9], fsc[9];
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) ff[i] = el(f[i], kf);
-                    // momentum of the neighbour's v = (j + F/2) / rho
-                    const real mvx = fma_(real(0.5), el(Fx, kf), el(jx, kf));
-                    const real mvy = fma_(real(0.5), el(Fy, kf), el(jy, kf));
-                    column_extrapolate<real>(A, el(rho_own, kc), el(rho, kf), el(vx, kf), el(vy, kf), mvx, mvy, ff,
-                                             fsc);
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) set_el(fs[i], kc, fsc[i]);
-                }
-                real *const out = G.fout;
-                const IX oi = (IX)r * rstride + xa;  // slot of (xa, r) in plane 0
-                const bool y_inner = WALLS ? (r >= 2 && r <= ny - 3) : (r >= 1 && r <= ny - 2);
-                if (x_inner && y_inner) {
-                    if constexpr (CP == 1) {
-                        out[oi] = fs[0];
-                        out[oi + o1] = fs[1];
-                        out[oi + o2] = fs[2];
-                        out[oi + o3] = fs[3];
-                        out[oi + o4] = fs[4];
-                        out[oi + o5] = fs[5];
-                        out[oi + o6] = fs[6];
-                        out[oi + o7] = fs[7];
-                        out[oi + o8] = fs[8];
+                if (!done) {
+                    V fe[9];
+                    feq_pairs<V>(rho, mul_(mx, irho), mul_(my, irho), mx, my, fe);
+                    if (A.mrt) {
+                        mrt_relax<V, real>(A, f, fe, fs);
                     } else {
-                        // directions without an x component keep the pair together
-                        stp<V>(out + oi, fs[0]);
-                        stp<V>(out + oi + o2, fs[2]);
-                        stp<V>(out + oi + o4, fs[4]);
-                        out[oi + o1] = el(fs[1], 0); out[oi + o1 + 1] = el(fs[1], 1);
-                        out[oi + o3] = el(fs[3], 0); out[oi + o3 + 1] = el(fs[3], 1);
-                        out[oi + o5] = el(fs[5], 0); out[oi + o5 + 1] = el(fs[5], 1);
-                        out[oi + o6] = el(fs[6], 0); out[oi + o6 + 1] = el(fs[6], 1);
-                        out[oi + o7] = el(fs[7], 0); out[oi + o7 + 1] = el(fs[7], 1);
-                        out[oi + o8] = el(fs[8], 0); out[oi + o8 + 1] = el(fs[8], 1);
-                    }
-                } else {
 #pragma unroll
-                    for (int k = 0; k < CP; ++k) {
-                        const int xk = xa + k;
-                        const IX ok = oi + k;
-#pragma unroll
-                        for (int i = 0; i < 9; ++i) {
-                            const int ty = r + ey_(i);
-                            if (WALLS && (ty == 0 || ty == ny - 1)) {
-                                // half-way bounce-back into the opposite slot of this node
-                                out[ok + opp_(i) * P] = el(fs[i], k);
-                            } else {
-                                int tx = xk + ex_(i);
-                                if (PRES) {
-                                    if (tx < 0 || tx >= nx) continue;  // leaves through the column
-                                } else {
-                                    tx = tx < 0 ? tx + nx : (tx >= nx ? tx - nx : tx);
-                                }
-                                int tyw = ty;
-                                if (!WALLS) tyw = ty < 0 ? ty + ny : (ty >= ny ? ty - ny : ty);
-                                out[(IX)tyw * rstride + i * P + tx] = el(fs[i], k);
-                            }
-                        }
+                        for (int i = 0; i < 9; ++i) fs[i] = fma_(sub_(fe[i], f[i]), bcr<V>(A.inv_tau), f[i]);
                     }
                 }
-                acc.macc = add_(acc.macc, rho_own);
-                acc.range(rho);
+            }
+            if (anyp) {
+                // pressure column: extrapolate from the interior neighbour
+                // (CP = 1: this thread's values are the neighbour's; pairs:
+                // the other element of the pair)
+                const int kc = pin ? 0 : CP - 1, kf = (CP == 1) ? 0 : (pin ? 1 : CP - 2);
+                real ff[9], fsc[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) ff[i] = el(f[i], kf);
+                // momentum of the neighbour's v = (j + F/2) / rho
+                const real mvx = fma_(real(0.5), el(Fx, kf), el(jx, kf));
+                const real mvy = fma_(real(0.5), el(Fy, kf), el(jy, kf));
+                column_extrapolate<real>(A, el(rho_own, kc), el(rho, kf), el(vx, kf), el(vy, kf), mvx, mvy, ff,
+                                         fsc);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) set_el(fs[i], kc, fsc[i]);
+            }
+            real *const out = G.fout;
+            const IX oi = (IX)r * rstride + xa;  // slot of (xa, r) in plane 0
+            const bool y_inner = WALLS ? (r >= 2 && r <= ny - 3) : (r >= 1 && r <= ny - 2);
+            if (x_inner && y_inner) {
+                if constexpr (CP == 1) {
+                    out[oi] = fs[0];
+                    out[oi + o1] = fs[1];
+                    out[oi + o2] = fs[2];
+                    out[oi + o3] = fs[3];
+                    out[oi + o4] = fs[4];
+                    out[oi + o5] = fs[5];
+                    out[oi + o6] = fs[6];
+                    out[oi + o7] = fs[7];
+                    out[oi + o8] = fs[8];
+                } else {
+                    // directions without an x component keep the pair together
+                    stp<V>(out + oi, fs[0]);
+                    stp<V>(out + oi + o2, fs[2]);
+                    stp<V>(out + oi + o4, fs[4]);
+                    out[oi + o1] = el(fs[1], 0); out[oi + o1 + 1] = el(fs[1], 1);
+                    out[oi + o3] = el(fs[3], 0); out[oi + o3 + 1] = el(fs[3], 1);
+                    out[oi + o5] = el(fs[5], 0); out[oi + o5 + 1] = el(fs[5], 1);
+                    out[oi + o6] = el(fs[6], 0); out[oi + o6 + 1] = el(fs[6], 1);
+                    out[oi + o7] = el(fs[7], 0); out[oi + o7 + 1] = el(fs[7], 1);
+                    out[oi + o8] = el(fs[8], 0); out[oi + o8 + 1] = el(fs[8], 1);
+                }
             } else {
 #pragma unroll
                 for (int k = 0; k < CP; ++k) {
-                    const bool pk = (k == 0 && pin) || (k == CP - 1 && pout);
-                    const int kv = (CP == 1 || !pk) ? k : (k == 0 ? 1 : CP - 2);  // a column reports v_f
-                    const long long oi = (long long)r * nx + xa + k;
-                    A.o_rho[oi] = el(rho_own, k);
-                    A.o_vx[oi] = el(vx, kv);
-                    A.o_vy[oi] = el(vy, kv);
+                    const int xk = xa + k;
+                    const IX ok = oi + k;
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) {
+                        const int ty = r + ey_(i);
+                        if (WALLS && (ty == 0 || ty == ny - 1)) {
+                            // half-way bounce-back into the opposite slot of this node
+                            out[ok + opp_(i) * P] = el(fs[i], k);
+                        } else {
+                            int tx = xk + ex_(i);
+                            if (PRES) {
+                                if (tx < 0 || tx >= nx) continue;  // leaves through the column
+                            } else {
+                                tx = tx < 0 ? tx + nx : (tx >= nx ? tx - nx : tx);
+                            }
+                            int tyw = ty;
+                            if (!WALLS) tyw = ty < 0 ? ty + ny : (ty >= ny ? ty - ny : ty);
+                            out[(IX)tyw * rstride + i * P + tx] = el(fs[i], k);
+                        }
+                    }
                 }
             }
+            acc.macc = add_(acc.macc, rho_own);
+            acc.range(rho);
 
             if (WALLS && (r <= 2 || r >= ny - 3)) {
                 // wall shear: quadratic through v = 0 on the half-way plane and
@@ -1146,32 +1133,25 @@ __device__ __forceinline__ void run_segment(const KArgs<real> &A, const Geom<rea
                 for (int k = 0; k < CP; ++k) {
                     const bool pk = (k == 0 && pin) || (k == CP - 1 && pout);
                     if (pk) continue;
-                    const int cc = ccol + k, xk = xa + k;
+                    const int cc = ccol + k;
                     const real rk = el(rho, k), vk = el(vx, k);
                     if (r == 1) {
                         b_rho1[k] = rk;
                         b_v1[k] = vk;
                         const real pw = wall_pressure<real, SW>(A, S.rho, S.phi, S.lap[q0][cc], qm, q0, qp, cc, rk);
-                        if (MODE == MODE_STEP) { acc.pmin = fmin(acc.pmin, pw); acc.pmax = fmax(acc.pmax, pw); }
-                        else A.o_pw[xk] = pw;
+                        acc.pmin = fmin(acc.pmin, pw); acc.pmax = fmax(acc.pmax, pw);
                     }
                     if (r == ny - 3) t_v2[k] = vk;
                     if (r == 2) {
                         const real tw = mul_(mul_(b_rho1[k], A.nu), mul_(fma_(real(9), b_v1[k], -vk), third));
-                        if (MODE == MODE_STEP) { acc.J += (double)tw; acc.tmin = fmin(acc.tmin, tw); acc.tmax = fmax(acc.tmax, tw); }
-                        else A.o_tw[xk] = tw;
+                        acc.J += (double)tw; acc.tmin = fmin(acc.tmin, tw); acc.tmax = fmax(acc.tmax, tw);
                     }
                     if (r == ny - 2) {
                         const real tw = mul_(mul_(rk, A.nu), mul_(fma_(real(9), vk, -t_v2[k]), third));
                         const real pw = wall_pressure<real, SW>(A, S.rho, S.phi, S.lap[q0][cc], qm, q0, qp, cc, rk);
-                        if (MODE == MODE_STEP) {
-                            acc.J += (double)tw;
-                            acc.tmin = fmin(acc.tmin, tw); acc.tmax = fmax(acc.tmax, tw);
-                            acc.pmin = fmin(acc.pmin, pw); acc.pmax = fmax(acc.pmax, pw);
-                        } else {
-                            A.o_tw[nx + xk] = tw;
-                            A.o_pw[nx + xk] = pw;
-                        }
+                        acc.J += (double)tw;
+                        acc.tmin = fmin(acc.tmin, tw); acc.tmax = fmax(acc.tmax, tw);
+                        acc.pmin = fmin(acc.pmin, pw); acc.pmax = fmax(acc.pmax, pw);
                     }
                 }
             }
@@ -1242,7 +1222,7 @@ __device__ __forceinline__ void cta_reduce(Acc<real, CP> &acc, SM &S, double &m,
 // arguments); otherwise the pitch is nx itself, which the compiler can share
 // with the bounds arithmetic (4% faster than carrying both). IX: the type of
 // population offsets, int while 9 pitch ny < 2^31, long long above.
-template <typename real, bool WALLS, bool PRES, int MODE, bool STAGED, bool PADDED, typename IX = int>
+template <typename real, bool WALLS, bool PRES, bool STAGED, bool PADDED, typename IX = int>
 __global__ void __launch_bounds__(threads_per_cta<real, STAGED>(),
                                   MinBlocks<real, threads_per_cta<real, STAGED>()>::value)
     step_kernel(const KArgs<real> A)
@@ -1281,12 +1261,11 @@ __global__ void __launch_bounds__(threads_per_cta<real, STAGED>(),
         const long long ue = min(u1, run_end);
         const int yb = ya + (int)(ue - u);
         u = ue;
-        run_segment<real, WALLS, PRES, MODE, BLOCK, STAGED, CP, PADDED, IX>(A, G, s, ya, yb, S, stages, bars, ring_next,
+        run_segment<real, WALLS, PRES, BLOCK, STAGED, CP, PADDED, IX>(A, G, s, ya, yb, S, stages, bars, ring_next,
                                                                        acc, lost);
     }
 
     if (STAGED && lost) atomicOr(A.err, 2);
-    if (MODE != MODE_STEP) return;
 
     double m, j;
     real e[4];
@@ -1354,7 +1333,7 @@ __global__ void __launch_bounds__(threads_per_cta<real, STAGED>(),
                            ch.rho_in_g, ch.rho_in_l, ch.rho_out_g, ch.rho_out_l};
         Acc<real, CP> acc;
         acc.reset();
-        run_segment<real, WALLS, PRES, MODE_STEP, BLOCK, STAGED, CP, true>(A, G, sg.strip, sg.ya, sg.yb, S, stages,
+        run_segment<real, WALLS, PRES, BLOCK, STAGED, CP, true>(A, G, sg.strip, sg.ya, sg.yb, S, stages,
                                                                           bars, ring_next, acc, lost);
         double m, j;
         real e[4];

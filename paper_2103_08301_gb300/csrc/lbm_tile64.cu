@@ -1,7 +1,8 @@
-// The FP64 step and fields by tiles (lbm_tile64.cuh): plan and launch.
+// The FP64 step and the fields by tiles (lbm_tile64.cuh): plan and launch.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdint>
 
 #include "lbm.h"
 #include "lbm_internal.h"
@@ -12,18 +13,22 @@ namespace lbm {
 
 namespace {
 
-template <int MODE, typename IX>
+template <typename real, int MODE, typename IX>
 void *pick(bool walls, bool pres)
 {
-    if (walls && pres) return (void *)step_kernel_tile64<true, true, MODE, IX>;
-    if (walls) return (void *)step_kernel_tile64<true, false, MODE, IX>;
-    if (pres) return (void *)step_kernel_tile64<false, true, MODE, IX>;
-    return (void *)step_kernel_tile64<false, false, MODE, IX>;
+    if (walls && pres) return (void *)step_kernel_tile64<real, true, true, MODE, IX>;
+    if (walls) return (void *)step_kernel_tile64<real, true, false, MODE, IX>;
+    if (pres) return (void *)step_kernel_tile64<real, false, true, MODE, IX>;
+    return (void *)step_kernel_tile64<real, false, false, MODE, IX>;
 }
-void *kernel(int mode, bool walls, bool pres, bool big)
+template <typename real>
+void *fields_kernel(bool walls, bool pres, bool big)
 {
-    if (mode == MODE_STEP) return big ? pick<MODE_STEP, long long>(walls, pres) : pick<MODE_STEP, int>(walls, pres);
-    return big ? pick<MODE_FIELDS, long long>(walls, pres) : pick<MODE_FIELDS, int>(walls, pres);
+    return big ? pick<real, MODE_FIELDS, long long>(walls, pres) : pick<real, MODE_FIELDS, int>(walls, pres);
+}
+void *step_kernel64(bool walls, bool pres, bool big)
+{
+    return big ? pick<double, MODE_STEP, long long>(walls, pres) : pick<double, MODE_STEP, int>(walls, pres);
 }
 
 }  // namespace
@@ -55,7 +60,7 @@ cudaError_t tile64_plan(int nx, int ny, bool walls, bool pres, bool big, int sms
     const long long ntiles = ntx * ((rows + p->sy + p->th - 1) / p->th);
     p->ntiles = (int)ntiles;
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel(MODE_STEP, walls, pres, big),
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, step_kernel64(walls, pres, big),
                                                                   T64_TX * p->th, 0);
     if (e != cudaSuccess) return e;
     p->ctas = (int)std::min<long long>(ntiles, std::min<long long>(MAX_CTAS, (long long)sms * std::max(1, occ)));
@@ -63,12 +68,93 @@ cudaError_t tile64_plan(int nx, int ny, bool walls, bool pres, bool big, int sms
     return cudaSuccess;
 }
 
-cudaError_t tile64_launch(const KArgs<double> &A, int mode, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
+cudaError_t tile64_launch(const KArgs<double> &A, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
                           cudaStream_t st)
 {
     T64Plan T{p.th, p.ntx, p.ntiles, p.sx, p.sy};
     void *args[] = {(void *)&A, (void *)&T};
-    return cudaLaunchKernel(kernel(mode, walls, pres, big), dim3(ctas), dim3(p.threads), args, 0, st);
+    return cudaLaunchKernel(step_kernel64(walls, pres, big), dim3(ctas), dim3(p.threads), args, 0, st);
 }
+
+namespace {
+
+// Whether a kernel may write `bytes` at p itself: memory of the current device,
+// aligned to its elements.
+bool writable_here(const void *p, size_t align)
+{
+    cudaPointerAttributes at{};
+    int dev = 0;
+    if ((uintptr_t)p % align != 0 || cudaGetDevice(&dev) != cudaSuccess) return false;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+bool overlap(const void *a, size_t na, const void *b, size_t nb)
+{
+    return (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na;
+}
+
+}  // namespace
+
+template <typename real>
+void fields_route(FieldsOut<real> &o, int nx, int ny, const void *busy, size_t busy_bytes)
+{
+    const size_t N = (size_t)nx * ny * sizeof(real), W = 2 * (size_t)nx * sizeof(real);
+    o.scratch = 0;
+    for (int k = 0; k < 5; ++k) {
+        const size_t bytes = k < 3 ? N : W;
+        o.bytes[k] = bytes;
+        bool direct = o.dst[k] && writable_here(o.dst[k], sizeof(real)) && !overlap(o.dst[k], bytes, busy, busy_bytes);
+        for (int j = 0; direct && j < 5; ++j)
+            if (j != k && o.dst[j] && overlap(o.dst[k], bytes, o.dst[j], j < 3 ? N : W)) direct = false;
+        o.ptr[k] = direct ? (real *)o.dst[k] : nullptr;
+        o.offset[k] = o.scratch;
+        if (o.dst[k] && !direct) o.scratch += (bytes + 255) / 256 * 256;
+    }
+}
+
+template <typename real>
+cudaError_t fields_tiles(KArgs<real> A, const FieldsOut<real> &o, bool walls, bool pres, bool big, int sms, cudaStream_t st)
+{
+    if (!walls) {  // no wall loads
+        for (int k = 3; k < 5; ++k)
+            if (o.ptr[k]) {
+                const cudaError_t e = cudaMemsetAsync(o.ptr[k], 0, o.bytes[k], st);
+                if (e != cudaSuccess) return e;
+            }
+    }
+    A.fout = nullptr;
+    A.reverse = 0;
+    A.o_rho = o.ptr[0]; A.o_vx = o.ptr[1]; A.o_vy = o.ptr[2]; A.o_tw = o.ptr[3]; A.o_pw = o.ptr[4];
+    Tile64 p;
+    cudaError_t e = tile64_plan(A.nx, A.ny, walls, pres, big, sms, &p);
+    if (e != cudaSuccess) return e;
+    T64Plan T{p.th, p.ntx, p.ntiles, p.sx, p.sy};
+    void *args[] = {(void *)&A, (void *)&T};
+    // no per-CTA slots: enough CTAs for every SM's threads
+    const int ctas = (int)std::min<long long>(p.ntiles, (long long)sms * 8);
+    return cudaLaunchKernel(fields_kernel<real>(walls, pres, big), dim3(ctas), dim3(p.threads), args, 0, st);
+}
+
+template <typename real>
+cudaError_t fields_copy(const FieldsOut<real> &o, cudaStream_t st)
+{
+    for (int k = 0; k < 5; ++k)
+        if (o.dst[k] && o.dst[k] != (void *)o.ptr[k]) {
+            const cudaError_t e = cudaMemcpyAsync(o.dst[k], o.ptr[k], o.bytes[k], cudaMemcpyDefault, st);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
+}
+
+#define INST(real)                                                                                                     \
+    template void fields_route<real>(FieldsOut<real> &, int, int, const void *, size_t);                              \
+    template cudaError_t fields_tiles<real>(KArgs<real>, const FieldsOut<real> &, bool, bool, bool, int, cudaStream_t); \
+    template cudaError_t fields_copy<real>(const FieldsOut<real> &, cudaStream_t);
+INST(float)
+INST(double)
+#undef INST
 
 }  // namespace lbm

@@ -1,5 +1,5 @@
-// The FP64 step and fields by tiles of 32 columns by th rows, one node per
-// thread.
+// The FP64 step, and the fields in either precision, by tiles of 32 columns by
+// th rows, one node per thread.
 //
 // GB300 runs FP64 at 1/64 of the FP32 rate (two thread-instructions per clock
 // and SM), so an FP64 step is bound by each SM's FP64 pipe: what counts is the
@@ -16,6 +16,10 @@
 // phi and Laplacian on (32 + 2)(th + 2)). The node arithmetic is the same helper
 // sequence in the same order, so the kernels give identical results.
 //
+// The FP32 fields (density, velocity, wall loads of the current state) take the
+// same kernel: they read 36 B and write 12 B per node once, with no row
+// pipeline to fill.
+//
 // Phases, a barrier after each: (1) densities and phi; (2) Laplacian; (3) force,
 // collision, boundaries, push, diagnostics. CTAs stride over the tiles.
 #pragma once
@@ -25,13 +29,14 @@ namespace lbm {
 constexpr int T64_TX = 32, T64_MAX = 8;  // tile columns; most rows
 constexpr int T64_AW = T64_TX + 4, T64_BW = T64_TX + 2;
 
+template <typename real>
 struct SmemT64 {
-    double rho[T64_AW * (T64_MAX + 4)];
-    double phi[T64_BW * (T64_MAX + 2)];
-    double lap[T64_BW * (T64_MAX + 2)];
-    double wv[T64_TX * T64_MAX];  // v_x of the rows next to the walls
+    real rho[T64_AW * (T64_MAX + 4)];
+    real phi[T64_BW * (T64_MAX + 2)];
+    real lap[T64_BW * (T64_MAX + 2)];
+    real wv[T64_TX * T64_MAX];  // v_x of the rows next to the walls
     double red[T64_MAX][2];
-    double ext[T64_MAX][4];
+    real ext[T64_MAX][4];
     int bad;
 };
 
@@ -43,18 +48,18 @@ struct T64Plan {
 };
 
 // row pointers of a shared array as the 3 x 3 operands of the stencils
-template <int SW>
-__device__ __forceinline__ Row3<double> row3d(const double *a, int r, int c)
+template <int SW, typename real>
+__device__ __forceinline__ Row3<real> row3d(const real *a, int r, int c)
 {
-    const double *p = a + r * SW + c;
-    return Row3<double>{p[-1], p[0], p[1]};
+    const real *p = a + r * SW + c;
+    return Row3<real>{p[-1], p[0], p[1]};
 }
 
-template <bool WALLS, bool PRES, int MODE, typename IX>
-__global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const KArgs<double> A, const T64Plan T)
+template <typename real, bool WALLS, bool PRES, int MODE, typename IX>
+__global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const KArgs<real> A, const T64Plan T)
 {
-    using real = double;
-    __shared__ SmemT64 S;
+    static_assert(sizeof(real) == 8 || MODE == MODE_FIELDS, "the FP32 step has its own kernels");
+    __shared__ SmemT64<real> S;
     const int tid = threadIdx.x, tx = tid & (T64_TX - 1), ty = tid >> 5, th = T.th, tn = T64_TX * th;
     const int nx = A.nx, ny = A.ny, P = A.pitch, rstride = 9 * P;
     const int yf0 = WALLS ? 1 : 0, yf1 = WALLS ? ny - 1 : ny;  // fluid rows yf0 .. yf1-1
@@ -197,13 +202,31 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
                     if (!WALLS) y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
                     out[(IX)y * rstride + i * P + x] = fs[i];
                 }
-                acc.mass += rho_own;
+                if constexpr (MODE == MODE_STEP) acc.mass += rho_own;
                 acc.range(rho);
             } else {
-                const long long oi = (long long)r * nx + xa;
-                A.o_rho[oi] = rho_own;
-                A.o_vx[oi] = vx;
-                A.o_vy[oi] = vy;
+                // outputs may be absent; wall rows and the wall loads of a
+                // pressure column are zero
+                auto put = [&](real *o, int y, real v) {
+                    if (o) o[(long long)y * nx + xa] = v;
+                };
+                put(A.o_rho, r, rho_own);
+                put(A.o_vx, r, vx);
+                put(A.o_vy, r, vy);
+                if (WALLS && (r == 1 || r == ny - 2)) {
+#pragma unroll
+                    for (int side = 0; side < 2; ++side) {
+                        if (r != (side ? ny - 2 : 1)) continue;
+                        const int y = side ? ny - 1 : 0;
+                        put(A.o_rho, y, real(0));
+                        put(A.o_vx, y, real(0));
+                        put(A.o_vy, y, real(0));
+                        if (anyp) {
+                            put(A.o_tw, side, real(0));
+                            put(A.o_pw, side, real(0));
+                        }
+                    }
+                }
             }
             if (WALLS && wall_row) S.wv[tid] = vx;
         }
@@ -233,8 +256,8 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
                             acc.tmin = fmin(acc.tmin, tw); acc.tmax = fmax(acc.tmax, tw);
                             acc.pmin = fmin(acc.pmin, pw); acc.pmax = fmax(acc.pmax, pw);
                         } else {
-                            A.o_tw[side * nx + xa] = tw;
-                            A.o_pw[side * nx + xa] = pw;
+                            if (A.o_tw) A.o_tw[side * nx + xa] = tw;
+                            if (A.o_pw) A.o_pw[side * nx + xa] = pw;
                         }
                     }
                 }
@@ -242,7 +265,7 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
         }
         __syncthreads();  // the shared arrays serve the next tile
     }
-    if (MODE != MODE_STEP) return;
+    if constexpr (MODE == MODE_STEP) {
 
     // fixed-order reduction: lanes by butterflies, then the warps in order
     const int lane = tid & 31, warp = tid >> 5;
@@ -284,6 +307,7 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
         ex[0] = fmin(ex[0], e[0]); ex[1] = fmax(ex[1], e[1]);
         ex[2] = fmin(ex[2], e[2]); ex[3] = fmax(ex[3], e[3]);
         if (S.bad) atomicOr(A.err, 1);
+    }
     }
 }
 
