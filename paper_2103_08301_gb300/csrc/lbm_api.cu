@@ -363,10 +363,9 @@ lbm_status plan_launch(lbm_ctx *ctx)
     // bulk-copy staging needs 16-byte aligned row segments
     ctx->staged = ctx->allow_staged && (ctx->pitch % 4 == 0) && (W % 4 == 0);
     // row pairs: FP32 staged grids with strips of at most R2_W columns (a
-    // multiple of 4); with periodic x the wrapped halo columns are copied as
-    // one 16-byte group, which needs nx a multiple of 4
+    // multiple of 4)
     ctx->rows2 = ctx->allow_rows2 && ctx->staged && ctx->grid.precision == 32 &&
-                 lbm::cols_per_thread<float, true>() == 1 && (ctx->grid.bc_x || nx % 4 == 0);
+                 lbm::cols_per_thread<float, true>() == 1;
     if (ctx->rows2) {
         const int W2 = lbm::strip_width(nx, std::min(wmax, lbm::R2_W), ctx->grid.bc_x);
         if (W2 % 4 == 0) W = W2;

@@ -14,9 +14,9 @@
 //     x0-4 .. x0+W+3), so the halo densities are summed from shared memory;
 //   - one producer thread stages each stencil row with a single 2-D tensor
 //     (TMA) load of 132 columns by 9 planes (cp.async.bulk.tensor through
-//     the tensor-map kernel parameter); strips whose halo wraps around a
-//     periodic x take nine plane copies and the wrap copies instead (plain
-//     cp.async.bulk). The batch kernel can read its channels' maps from
+//     the tensor-map kernel parameter); in a batch, strips whose halo wraps
+//     around a periodic x take nine plane copies and the wrap copies instead
+//     (plain cp.async.bulk). The batch kernel can read its channels' maps from
 //     device memory, but by default it takes the plane copies (faster there:
 //     58.9k against 56.3k MLUPS on the 64-channel sweep). Nine copies per row in
 //     place of one load cost 7% of the step;
@@ -30,9 +30,11 @@
 //       yy0-1, yy0 on local columns -1 .. xw;              --- barrier B ---
 //   (3) force, collision, boundaries and push of rows yy0-2, yy0-1 (pair k-1,
 //       k >= 2; the second row only if it is below yb).
-// Restricted to strips and pitches that are multiples of 4 and, with periodic
-// x, to nx a multiple of 4 (the wrapped halo columns are copied as one
-// 16-byte group from each end of the row).
+// Restricted to strips and pitches that are multiples of 4; a batch with
+// periodic x also to nx a multiple of 4 (its wrapped halo columns are copied as
+// one 16-byte group from each end of the row). A single channel's wrapped halo
+// lanes copy their own columns: a periodic width that is not a multiple of 4 ran
+// the one-row kernel before (1999 x 1501, Peng-Robinson, MRT: 71 us a step).
 #pragma once
 
 namespace lbm {
@@ -107,6 +109,19 @@ __device__ __forceinline__ Row3<float2> row3p(const float (*S)[SW], int ra, int 
 
 // Static shared memory of a row-pair CTA: the 8-row rings of density, phi
 // and Laplacian (one column per lane) and the reduction scratch.
+// Populations of the wrapped halo columns (periodic x), by pair slot, row, plane
+// and the lanes -2, -1, xw, xw+1 that hold them.
+struct WrapR2 {
+    float v[R2_SLOTS][2][9][4];
+};
+// Asynchronous 4-byte copy into shared memory by the generic proxy; each lane
+// waits for its own copies and reads only what it copied.
+__device__ __forceinline__ void cp_async4(void *dst, const float *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 struct SmemR2 {
     __align__(16) float rho[RING][R2_BLOCK + 4];
     __align__(16) float phi[RING][R2_BLOCK + 4];
@@ -135,12 +150,17 @@ __device__ __forceinline__ float2 stage_pair(const float *slot, int i, int sc)
 // left in flight when the CTA exits.
 // EARLY: stencil-row pairs issued together when a segment starts (1 .. the
 // three slots, all free then); later pairs are issued one per iteration.
-template <bool WALLS, bool PRES, bool PADDED, bool HOOK = false, typename IX = int, int EARLY = 1>
+// DIRECT (periodic x): the halo lanes beyond either end of the row copy their
+// wrapped columns themselves, 4 bytes at a time, into `wrap`: any width, and
+// every strip on tensor loads. Without it (the batch) the wrapped columns come as
+// one 16-byte bulk copy from each end, for which nx is a multiple of 4.
+template <bool WALLS, bool PRES, bool PADDED, bool HOOK = false, typename IX = int, int EARLY = 1, bool DIRECT = false>
 __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom<float> &G, int s, int ya, int yb,
                                                SmemR2 &S, float *stages, uint64_t *bars,
                                                RingPos2 &ring_next, const CUtensorMap *tmap, Acc<float, 1> &acc,
-                                               bool &lost, bool skip_here)
+                                               bool &lost, bool skip_here, WrapR2 *wrap = nullptr)
 {
+    static_assert(!(DIRECT && PRES), "pressure columns have no wrapped halo");
     using V = float2;
     constexpr int SW = R2_BLOCK + 4;
     constexpr int PRODUCER = R2_BLOCK - 1;  // no halo duty
@@ -188,7 +208,10 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
     const int gx0 = max(x0 - 4, 0);
     const int gx1 = min(x0 + xw + 4, G.pitch);
     const uint32_t mbytes = (uint32_t)((gx1 - gx0) * sizeof(float));
-    const bool wrapL = !PRES && x0 == 0, wrapR = !PRES && x0 + xw == nx;
+    const bool wrapL = !PRES && !DIRECT && x0 == 0, wrapR = !PRES && !DIRECT && x0 + xw == nx;
+    // DIRECT: this lane's column lies beyond an end of the row, at wcol
+    const bool wrapped = DIRECT && dens && (g < 0 || g >= nx);
+    const int wcol = wrapped ? ((g % nx) + nx) % nx : 0, wlane = l < 0 ? l + 2 : l - xw + 2;
     const uint32_t row_bytes = 9u * (mbytes + (wrapL ? 16u : 0u) + (wrapR ? 16u : 0u));
     const int dcol = gx0 - x0 + 4;
     const int npairs = (yb - ya + 5) / 2;  // stencil rows ya-2 .. yb+1 in pairs
@@ -215,6 +238,17 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
             if (q == 0)
                 for (int d = 1; d < A.pf; ++d) prefetch(d);
             prefetch(q + A.pf);
+        }
+        if constexpr (DIRECT) {
+            if (wrapped && q < npairs) {
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    bool mir;
+                    const float *src = G.fin + (IX)map_row<WALLS>(ya - 2 + 2 * q + t, ny, mir) * rstride + wcol;
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) cp_async4(&wrap->v[ring_issue.s][t][i][wlane], src + i * P);
+                }
+            }
         }
         if (q < npairs) {
             if (HOOK && skip_here && q == npairs - 1) {
@@ -278,6 +312,14 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
                 V pf[9];
 #pragma unroll
                 for (int i = 0; i < 9; ++i) pf[i] = stage_pair(slot, i, dsc);
+                if constexpr (DIRECT) {
+                    if (wrapped) {
+                        cp_async_wait_all();
+#pragma unroll
+                        for (int i = 0; i < 9; ++i)
+                            pf[i] = make_float2(wrap->v[cur][0][i][wlane], wrap->v[cur][1][i][wlane]);
+                    }
+                }
                 V sum = add_(add_(add_(pf[0], pf[1]), add_(pf[2], pf[3])), add_(add_(pf[4], pf[5]), add_(pf[6], pf[7])));
                 sum = add_(sum, pf[8]);
                 if (dmode) {
@@ -466,6 +508,9 @@ __global__ void __launch_bounds__(R2_BLOCK, LBM_R2_MIN_BLOCKS)
     float *const stages = reinterpret_cast<float *>(dsm);
     uint64_t *const bars = reinterpret_cast<uint64_t *>(dsm + (size_t)R2_SLOTS * R2_SLOT * sizeof(float));
     __shared__ SmemR2 S;
+    constexpr bool DIRECT = !PRES;
+    __shared__ WrapR2 wrap_s;
+    WrapR2 *const wrap = DIRECT ? &wrap_s : nullptr;
 
     const int tid = threadIdx.x;
     const int cta = A.reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
@@ -496,8 +541,9 @@ __global__ void __launch_bounds__(R2_BLOCK, LBM_R2_MIN_BLOCKS)
         const int yb = ya + (int)(ue - u);
         u = ue;
         // the test hook applies to the first CTA's last segment
-        run_segment_r2<WALLS, PRES, PADDED, HOOK, IX, EARLY>(A, G, s, ya, yb, S, stages, bars, ring_next,
-                                                  A.tma ? &tmap : nullptr, acc, lost, HOOK && cta == 0 && u == u1);
+        run_segment_r2<WALLS, PRES, PADDED, HOOK, IX, EARLY, DIRECT>(
+            A, G, s, ya, yb, S, stages, bars, ring_next, A.tma ? &tmap : nullptr, acc, lost,
+            HOOK && cta == 0 && u == u1, wrap);
     }
     if (lost) atomicOr(A.err, 2);
 
