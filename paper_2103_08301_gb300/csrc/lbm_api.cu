@@ -137,6 +137,7 @@ struct lbm_ctx {
     // general wall geometry (lbm_mask.cu): set when the mask adds solid nodes
     // to the wall rows, or when LBM_OPT_GENERAL forces that path
     lbm::MaskPath *mask = nullptr;
+    bool mask_rows2 = false;  // its FP32 step by row pairs, over the row-pair plan
     std::vector<uint8_t> mask_host;  // the caller's mask (empty: none)
     bool force_general = false;
     bool fault_skip = false;  // LBM_OPT_FAULT_SKIP_COPY (test hook)
@@ -560,8 +561,17 @@ lbm_status one_step(lbm_ctx *ctx)
         ctx->step += 1;
         return LBM_OK;
     }
-    cudaError_t e = ctx->mask ? lbm::mask_launch<real>(ctx->mask, A, lbm::MODE_STEP, ctx->stream)
-                              : launch<real>(ctx, A);
+    cudaError_t e;
+    if (!ctx->mask) {
+        e = launch<real>(ctx, A);
+    } else if (sizeof(real) == 4 && ctx->mask_rows2) {
+        lbm::KArgs<float> B = make_args<float>(ctx);
+        B.tma = ctx->tma_ok && ctx->allow_tma;
+        B.pf = ctx->pf;
+        e = lbm::mask_rows2_launch(ctx->mask, B, &ctx->tmap[ctx->cur], ctx->early, ctx->stream);
+    } else {
+        e = lbm::mask_launch<real>(ctx->mask, A, lbm::MODE_STEP, ctx->stream);
+    }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "step launch");
     ctx->cur = 1 - ctx->cur;
     ctx->step += 1;
@@ -736,7 +746,17 @@ lbm_status plan_geometry(lbm_ctx *ctx)
     }
     lbm_status st = lbm::mask_setup(m, ctx->grid, ctx->pitch, ctx->sms, ctx->force_general, ctx->stream, &ctx->mask,
                                     ctx->last_error, sizeof ctx->last_error);
-    if (st == LBM_OK && ctx->mask) ctx->nctas = lbm::mask_blocks(ctx->mask);
+    ctx->mask_rows2 = false;
+    if (st != LBM_OK || !ctx->mask) return st;
+    if (ctx->rows2 && !ctx->big) {
+        // the row-pair plan holds where as many CTAs stay resident
+        int per_sm = 0;
+        cudaError_t e = lbm::mask_rows2_plan(ctx->mask, ctx->early, &per_sm);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "mask step plan");
+        ctx->mask_rows2 = true;
+        return LBM_OK;
+    }
+    ctx->nctas = lbm::mask_blocks(ctx->mask);
     return st;
 }
 

@@ -104,6 +104,11 @@ void mask_free(MaskPath *m);
 int mask_blocks(const MaskPath *m);  // CTAs of the collide kernel (diagnostic slots)
 template <typename real>
 cudaError_t mask_launch(const MaskPath *m, const KArgs<real> &A, int mode, cudaStream_t stream);
+// The FP32 step by row pairs over the caller's plan (A.nctas CTAs, strips of
+// A.W; map: tensor map of A.fin), and its resident CTAs per SM.
+cudaError_t mask_rows2_plan(const MaskPath *m, bool early, int *ctas_per_sm);
+cudaError_t mask_rows2_launch(const MaskPath *m, const KArgs<float> &A, const CUtensorMap *map, bool early,
+                              cudaStream_t stream);
 
 // In-place streaming (the AA pattern) of a single context (lbm_inplace.cu):
 // one population array F, a density plane rho (pitch * ny) and a side buffer

@@ -18,6 +18,14 @@
 // The ghost sources are resolved on the host into a table of fluid (or
 // pressure-column) nodes per ghost point, so one gather per point fills them.
 //
+// FP32 steps (where the row-pair plan applies): two kernels. The ghost densities
+// of the solid points within reach of the fluid are gathered, each from its few
+// sources' populations, and the row-pair kernel (lbm_rows2.cuh, MASK) does the
+// step with them, reading per point a 16-bit word of link and ghost flags: 74 B
+// per node and the rows around the obstacles instead of the 130 below. The 4096 x
+// 1024 channel with constrictions: 170 us a step in the six kernels below (which
+// remain for FP64, the fields and grids without row pairs), 107 us in these two.
+//
 // Data (device, allocated by the library): the solid mask (1 B/node), three
 // ghost-extended arrays of (nx + 4)(ny + 4) values (density, phi, Laplacian),
 // the ghost table, and the wall-row velocities and pressures of the
@@ -53,6 +61,12 @@ struct MaskDev {
     const int *gdst, *gbeg, *gsrc;        // ghost table (CSR)
     const uint8_t *gwet;
     int nghost;
+    // FP32 row pairs: flags of every extended point (bit 15: the density is a
+    // ghost; bits 1-8 of a lattice node: links that bounce back) and the ghosts
+    // with sources, sources as lattice nodes
+    const uint16_t *xflags;
+    const int *fdst, *fbeg, *fsrc;
+    int nfast;
 };
 
 __device__ __forceinline__ int ext(const MaskDev &m, int x, int y) { return (y + 2) * m.sx + (x + 2); }
@@ -103,6 +117,79 @@ __global__ void __launch_bounds__(MB) mask_ghost_kernel(const KArgs<real> A, con
             v = add_(s, m.gwet[k] ? A.wet : real(0));
         }
         E[m.gdst[k]] = v;
+    }
+}
+
+// Ghost densities for the row-pair step: the mean of the sources' densities, each
+// summed from its populations (a pressure column's from its interior neighbour).
+__global__ void __launch_bounds__(MB) mask_fast_ghost_kernel(const KArgs<float> A, const MaskDev m, float *E)
+{
+    const Geom<float> G{A.fin, A.fout, A.nx, A.ny, A.W, A.pitch, A.rho_in_g, A.rho_in_l, A.rho_out_g, A.rho_out_l};
+    for (int k = blockIdx.x * MB + threadIdx.x; k < m.nfast; k += gridDim.x * MB) {
+        const int b = m.fbeg[k], e = m.fbeg[k + 1];
+        float s = 0.f;
+        for (int j = b; j < e; ++j) {
+            const int node = m.fsrc[j], y = node / m.nx, x = node - y * m.nx;
+            const bool pin = m.bc_x && x == 0, pout = m.bc_x && x == m.nx - 1;
+            float v = pop_sum<float>(A.fin, y * 9 * m.pitch + (pin ? 1 : (pout ? m.nx - 2 : x)), m.pitch);
+            if (pin || pout) v = add_(column_density(A, G, pout, v), 0.f);
+            s = j == b ? v : add_(s, v);
+        }
+        if (e - b > 1) s = s / (float)(e - b);
+        E[m.fdst[k]] = add_(s, A.wet);
+    }
+}
+
+// The row-pair step with solid nodes (lbm_rows2.cuh); launched like
+// step_kernel_rows2.
+template <bool WALLS, bool PRES, int EARLY>
+__global__ void __launch_bounds__(R2_BLOCK, LBM_R2_MIN_BLOCKS)
+    mask_step_kernel_rows2(const KArgs<float> A, const __grid_constant__ CUtensorMap tmap, const MaskR2 mk)
+{
+    extern __shared__ __align__(128) unsigned char dsm[];
+    float *const stages = reinterpret_cast<float *>(dsm);
+    uint64_t *const bars = reinterpret_cast<uint64_t *>(dsm + (size_t)R2_SLOTS * R2_SLOT * sizeof(float));
+    __shared__ SmemR2 S;
+    __shared__ WrapR2 wrap_s;
+    constexpr bool DIRECT = !PRES;
+
+    const int tid = threadIdx.x;
+    const int cta = A.reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+    long long u = cut_units<WALLS>(A, cta);
+    const long long u1 = cut_units<WALLS>(A, cta + 1);
+    const Geom<float> G{A.fin, A.fout, A.nx, A.ny, A.W, A.pitch, A.rho_in_g, A.rho_in_l, A.rho_out_g, A.rho_out_l};
+    Acc<float, 1> acc;
+    acc.reset();
+    RingPos2 ring_next;
+    bool lost = false;
+    if (tid == 0) {
+        for (int st = 0; st < R2_SLOTS; ++st) mbar_init(&bars[st], 1);
+        mbar_init_fence();
+    }
+    __syncthreads();
+    while (u < u1) {
+        int s, ya;
+        long long run_end;
+        unit_run(A, u, s, ya, run_end);
+        const long long ue = min(u1, run_end);
+        const int yb = ya + (int)(ue - u);
+        u = ue;
+        run_segment_r2<WALLS, PRES, true, false, int, EARLY, DIRECT, true>(
+            A, G, s, ya, yb, S, stages, bars, ring_next, A.tma ? &tmap : nullptr, acc, lost, false,
+            DIRECT ? &wrap_s : nullptr, mk);
+    }
+    if (lost) atomicOr(A.err, 2);
+    double m, j;
+    float e[4];
+    bool anybad;
+    cta_reduce<float, R2_BLOCK, 1>(acc, S, m, j, e, anybad);
+    if (tid == 0) {
+        A.mass_part[cta] = m;
+        A.J_acc[cta] += j;
+        float *ex = A.ext + 4 * cta;
+        ex[0] = fmin(ex[0], e[0]); ex[1] = fmax(ex[1], e[1]);
+        ex[2] = fmin(ex[2], e[2]); ex[3] = fmax(ex[3], e[3]);
+        if (anybad) atomicOr(A.err, 1);
     }
 }
 
@@ -457,6 +544,25 @@ lbm_status mask_setup(const uint8_t *mask, const lbm_grid &g, int pitch, int sms
             links[(size_t)y * nx + x] = l;
         }
 
+    // FP32 row pairs: flags per extended point, ghosts with sources
+    std::vector<uint16_t> xflags;
+    std::vector<int> fdst, fbeg{0}, fsrc;
+    if (g.precision == 32) {
+        xflags.assign((size_t)(nx + 4) * (ny + 4), 0);
+        for (int y = 0; y < ny; ++y)
+            for (int x = 0; x < nx; ++x) xflags[ext_idx(x, y)] = links[(size_t)y * nx + x];
+        for (size_t k = 0; k < gdst.size(); ++k) {
+            xflags[gdst[k]] = gwet[k] ? (uint16_t)0x8000u : (uint16_t)0;
+            if (!gwet[k] || gbeg[k + 1] == gbeg[k]) continue;
+            fdst.push_back(gdst[k]);
+            for (int j = gbeg[k]; j < gbeg[k + 1]; ++j) {
+                const int ey = gsrc[j] / sx - 2, ex = gsrc[j] % sx - 2;
+                fsrc.push_back(ey * nx + ex);
+            }
+            fbeg.push_back((int)fsrc.size());
+        }
+    }
+
     MaskPath *m = new (std::nothrow) MaskPath();
     if (!m) return LBM_ERR_OOM;
     m->precision = g.precision;
@@ -466,8 +572,10 @@ lbm_status mask_setup(const uint8_t *mask, const lbm_grid &g, int pitch, int sms
     const size_t b_solid = al(solid.size()), b_links = al(links.size() * 2), b_ext = al(m->ne * sz),
                  b_dst = al(gdst.size() * 4),
                  b_beg = al(gbeg.size() * 4), b_src = al(std::max<size_t>(1, gsrc.size()) * 4),
-                 b_wet = al(gwet.size()), b_wv = al(4 * (size_t)nx * sz), b_pw = al(2 * (size_t)nx * sz);
-    const size_t total = b_solid + b_links + 3 * b_ext + b_dst + b_beg + b_src + b_wet + b_wv + b_pw;
+                 b_xf = al(xflags.size() * 2), b_fdst = al(fdst.size() * 4), b_fbeg = al(fbeg.size() * 4),
+                 b_fsrc = al(fsrc.size() * 4), b_wet = al(gwet.size()), b_wv = al(4 * (size_t)nx * sz), b_pw = al(2 * (size_t)nx * sz);
+    const size_t total = b_solid + b_links + 3 * b_ext + b_dst + b_beg + b_src + b_wet + b_wv + b_pw +
+                         b_xf + b_fdst + b_fbeg + b_fsrc;
     if (cudaMalloc((void **)&m->mem, total) != cudaSuccess) {
         cudaGetLastError();
         delete m;
@@ -484,7 +592,11 @@ lbm_status mask_setup(const uint8_t *mask, const lbm_grid &g, int pitch, int sms
     int *d_src = (int *)p; p += b_src;
     uint8_t *d_wet = p; p += b_wet;
     m->wv = p; p += b_wv;
-    m->pw = p;
+    m->pw = p; p += b_pw;
+    uint16_t *d_xf = (uint16_t *)p; p += b_xf;
+    int *d_fdst = (int *)p; p += b_fdst;
+    int *d_fbeg = (int *)p; p += b_fbeg;
+    int *d_fsrc = (int *)p;
     cudaError_t e = cudaMemsetAsync(m->mem, 0, total, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_solid, solid.data(), solid.size(), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess)
@@ -494,6 +606,13 @@ lbm_status mask_setup(const uint8_t *mask, const lbm_grid &g, int pitch, int sms
     if (e == cudaSuccess && !gsrc.empty())
         e = cudaMemcpyAsync(d_src, gsrc.data(), gsrc.size() * 4, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_wet, gwet.data(), gwet.size(), cudaMemcpyHostToDevice, stream);
+    auto up = [&](void *dst, const void *src, size_t bytes) {
+        if (e == cudaSuccess && bytes > 0) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, stream);
+    };
+    up(d_xf, xflags.data(), xflags.size() * 2);
+    up(d_fdst, fdst.data(), fdst.size() * 4);
+    up(d_fbeg, fbeg.data(), fbeg.size() * 4);
+    up(d_fsrc, fsrc.data(), fsrc.size() * 4);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // the host vectors die here
     if (e != cudaSuccess) {
         std::snprintf(err, errlen, "wall mask upload: %s", cudaGetErrorString(e));
@@ -501,7 +620,7 @@ lbm_status mask_setup(const uint8_t *mask, const lbm_grid &g, int pitch, int sms
         return LBM_ERR_CUDA;
     }
     m->d = MaskDev{nx, ny, pitch, g.walls, g.bc_x, sx, d_solid, d_links, d_dst, d_beg, d_src, d_wet,
-                   (int)gdst.size()};
+                   (int)gdst.size(), d_xf, d_fdst, d_fbeg, d_fsrc, (int)fdst.size()};
     const long long nodes = (long long)nx * ny;
     m->blocks = (int)std::max<long long>(1, std::min<long long>((nodes + MB - 1) / MB, (long long)sms * 8));
     m->blocks = std::min(m->blocks, MAX_CTAS);
@@ -512,6 +631,36 @@ lbm_status mask_setup(const uint8_t *mask, const lbm_grid &g, int pitch, int sms
 namespace {
 int grid_for(long long n, int cap) { return (int)std::max<long long>(1, std::min<long long>((n + MB - 1) / MB, cap)); }
 }  // namespace
+
+namespace {
+template <int EARLY>
+void *rows2_ptr(bool walls, bool pres)
+{
+    if (walls && pres) return (void *)mask_step_kernel_rows2<true, true, EARLY>;
+    if (walls) return (void *)mask_step_kernel_rows2<true, false, EARLY>;
+    if (pres) return (void *)mask_step_kernel_rows2<false, true, EARLY>;
+    return (void *)mask_step_kernel_rows2<false, false, EARLY>;
+}
+}  // namespace
+
+cudaError_t mask_rows2_plan(const MaskPath *m, bool early, int *ctas_per_sm)
+{
+    void *fn = early ? rows2_ptr<3>(m->d.walls, m->d.bc_x) : rows2_ptr<1>(m->d.walls, m->d.bc_x);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows2_smem_bytes());
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, fn, R2_BLOCK, rows2_smem_bytes());
+    return e;
+}
+
+cudaError_t mask_rows2_launch(const MaskPath *m, const KArgs<float> &A, const CUtensorMap *map, bool early, cudaStream_t s)
+{
+    float *E = (float *)m->E;
+    if (m->d.nfast > 0) mask_fast_ghost_kernel<<<grid_for(m->d.nfast, m->blocks), MB, 0, s>>>(A, m->d, E);
+    const MaskR2 mk{m->d.xflags, E, m->d.sx};
+    void *fn = early ? rows2_ptr<3>(m->d.walls, m->d.bc_x) : rows2_ptr<1>(m->d.walls, m->d.bc_x);
+    void *args[] = {(void *)&A, (void *)map, (void *)&mk};
+    return cudaLaunchKernel(fn, dim3(A.nctas), dim3(R2_BLOCK), args, rows2_smem_bytes(), s);
+}
 
 template <typename real>
 cudaError_t mask_launch(const MaskPath *m, const KArgs<real> &A, int mode, cudaStream_t s)

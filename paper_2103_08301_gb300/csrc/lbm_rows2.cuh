@@ -150,15 +150,30 @@ __device__ __forceinline__ float2 stage_pair(const float *slot, int i, int sc)
 // left in flight when the CTA exits.
 // EARLY: stencil-row pairs issued together when a segment starts (1 .. the
 // three slots, all free then); later pairs are issued one per iteration.
+// General geometry (MASK): a lattice node's bounce-back links and, for every
+// point of the lattice extended by two nodes (row stride sx), whether its
+// density is a ghost (bit 15: solid, or behind a wall row) to be read from E.
+struct MaskR2 {
+    const uint16_t *flags;
+    const float *E;
+    int sx;
+};
+
+// MASK: the segment of a lattice with solid nodes (lbm_mask.cu): ghost densities
+// come from MaskR2::E, solid nodes neither collide nor count, pushes along a
+// marked link bounce back. Flags are read one pair ahead, ghost densities at the
+// end of the iteration before, so neither stands between a pair and its density.
 // DIRECT (periodic x): the halo lanes beyond either end of the row copy their
 // wrapped columns themselves, 4 bytes at a time, into `wrap`: any width, and
 // every strip on tensor loads. Without it (the batch) the wrapped columns come as
 // one 16-byte bulk copy from each end, for which nx is a multiple of 4.
-template <bool WALLS, bool PRES, bool PADDED, bool HOOK = false, typename IX = int, int EARLY = 1, bool DIRECT = false>
+template <bool WALLS, bool PRES, bool PADDED, bool HOOK = false, typename IX = int, int EARLY = 1, bool DIRECT = false,
+          bool MASK = false>
 __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom<float> &G, int s, int ya, int yb,
                                                SmemR2 &S, float *stages, uint64_t *bars,
                                                RingPos2 &ring_next, const CUtensorMap *tmap, Acc<float, 1> &acc,
-                                               bool &lost, bool skip_here, WrapR2 *wrap = nullptr)
+                                               bool &lost, bool skip_here, WrapR2 *wrap = nullptr,
+                                               const MaskR2 mk = MaskR2{})
 {
     static_assert(!(DIRECT && PRES), "pressure columns have no wrapped halo");
     using V = float2;
@@ -288,6 +303,20 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
         }
     };
 
+    // MASK: flags of the pairs k, k-1 (k-2's second row) and ghost densities of pair k
+    unsigned fc0 = 0, fc1 = 0, fp0 = 0, fp1 = 0, fq1 = 0;
+    float gh0 = 0.f, gh1 = 0.f;
+    const int mx = MASK ? min(max(g, -2), nx + 1) + 2 : 0;
+    auto ext_of = [&](int yy) { return min(yy + 2, ny + 3) * mk.sx + mx; };
+    if constexpr (MASK) {
+        if (dens) {
+            fc0 = mk.flags[ext_of(ya - 2)];
+            fc1 = mk.flags[ext_of(ya - 1)];
+            if (fc0 >> 15) gh0 = mk.E[ext_of(ya - 2)];
+            if (fc1 >> 15) gh1 = mk.E[ext_of(ya - 1)];
+        }
+    }
+
     // with EARLY > 1 the first pairs go out together, so only the first wait
     // of a segment sees the full latency of a stage load (short segments)
     static_assert(EARLY >= 1 && EARLY <= R2_SLOTS, "early pairs fit the free slots");
@@ -326,10 +355,21 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
                     sum.x = column_density(A, G, dmode == 3, sum.x);
                     sum.y = column_density(A, G, dmode == 3, sum.y);
                 }
-                const V rho_c = add_(sum, add);
+                V rho_c = add_(sum, add);
+                if constexpr (MASK) {
+                    if (fc0 >> 15) rho_c.x = gh0;
+                    if (fc1 >> 15) rho_c.y = gh1;
+                }
                 const V ph = eos_phi<V>(A, rho_c);
                 S.rho[r0][tid] = rho_c.x; S.rho[r1][tid] = rho_c.y;
                 S.phi[r0][tid] = ph.x; S.phi[r1][tid] = ph.y;
+            }
+        }
+        unsigned fn0 = 0, fn1 = 0;  // MASK: flags of pair k+1
+        if constexpr (MASK) {
+            if (dens && k + 1 < npairs) {
+                fn0 = mk.flags[ext_of(yy0 + 2)];
+                fn1 = mk.flags[ext_of(yy0 + 3)];
             }
         }
         __syncthreads();  // A: density rows complete; the slot of pair k-2 is free
@@ -353,6 +393,7 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
         if (k >= 2 && active) {
             const int b = yy0 - 2;
             const bool second = b + 1 < yb;
+            const bool s0 = MASK && (fp0 >> 15), s1 = MASK && (fp1 >> 15);  // solid nodes of the pair
             const float *slot = stages + (size_t)prev * R2_SLOT;
             V f[9];
 #pragma unroll
@@ -406,7 +447,7 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
             float *const out = G.fout;
             const IX oi = (IX)b * rstride + xa;  // slot of (xa, b) in plane 0
             const bool y_inner = WALLS ? (b >= 2 && b + 1 <= ny - 3) : (b >= 1 && b + 1 <= ny - 2);
-            if (x_inner && y_inner && second) {
+            if (x_inner && y_inner && second && !(MASK && (fp0 | fp1))) {
                 const IX oj = oi + rstride;
                 out[oi] = fs[0].x;      out[oj] = fs[0].y;
                 out[oi + o1] = fs[1].x; out[oj + o1] = fs[1].y;
@@ -421,12 +462,13 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     if (e == 1 && !second) break;
+                    if (e ? s1 : s0) continue;
                     const int r = b + e;
                     const IX ok = oi + (IX)e * rstride;
 #pragma unroll
                     for (int i = 0; i < 9; ++i) {
                         const int ty = r + ey_(i);
-                        if (WALLS && (ty == 0 || ty == ny - 1)) {
+                        if (MASK ? ((e ? fp1 : fp0) >> i) & 1u : WALLS && (ty == 0 || ty == ny - 1)) {
                             // half-way bounce-back into the opposite slot of this node
                             out[ok + opp_(i) * P] = el(fs[i], e);
                         } else {
@@ -445,14 +487,18 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
             }
             // diagnostics of the state read, row by row in the one-row kernel's
             // order (its flush follows collided row r when (r - ya + 5) % 16 == 15)
-            acc.macc = add_(acc.macc, rho_own.x);
-            acc.rmin = vmin_(acc.rmin, rho.x);
-            acc.rmax = vmax_(acc.rmax, rho.x);
+            if (!s0) {
+                acc.macc = add_(acc.macc, rho_own.x);
+                acc.rmin = vmin_(acc.rmin, rho.x);
+                acc.rmax = vmax_(acc.rmax, rho.x);
+            }
             if (((b - ya + 5) & 15) == 15) acc.flush();
             if (second) {
-                acc.macc = add_(acc.macc, rho_own.y);
-                acc.rmin = vmin_(acc.rmin, rho.y);
-                acc.rmax = vmax_(acc.rmax, rho.y);
+                if (!s1) {
+                    acc.macc = add_(acc.macc, rho_own.y);
+                    acc.rmin = vmin_(acc.rmin, rho.y);
+                    acc.rmax = vmax_(acc.rmax, rho.y);
+                }
                 if (((b + 1 - ya + 5) & 15) == 15) acc.flush();
             }
 
@@ -465,18 +511,21 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
                     const int r = b + e;
                     const float rk = el(rho, e), vk = el(vx, e);
                     const int pm = (r - 1) & RM, pz = r & RM, pp = (r + 1) & RM;
-                    if (r == 1) {
+                    // MASK: a wall column counts where both rows next to the wall
+                    // are fluid (rows 1 and 2 are one pair)
+                    const bool low = !MASK || !(s0 || s1), high = !MASK || !(e ? s0 || s1 : s0 || (fq1 >> 15) != 0);
+                    if (r == 1 && low) {
                         b_rho1 = rk;
                         b_v1 = vk;
                         const float pw = wall_pressure<float, SW>(A, S.rho, S.phi, S.lap[pz][ccol], pm, pz, pp, ccol, rk);
                         acc.pmin = fmin(acc.pmin, pw); acc.pmax = fmax(acc.pmax, pw);
                     }
                     if (r == ny - 3) t_v2 = vk;
-                    if (r == 2) {
+                    if (r == 2 && low) {
                         const float tw = mul_(mul_(b_rho1, A.nu), mul_(fma_(9.0f, b_v1, -vk), third));
                         acc.J += (double)tw; acc.tmin = fmin(acc.tmin, tw); acc.tmax = fmax(acc.tmax, tw);
                     }
-                    if (r == ny - 2) {
+                    if (r == ny - 2 && high) {
                         const float tw = mul_(mul_(rk, A.nu), mul_(fma_(9.0f, vk, -t_v2), third));
                         const float pw = wall_pressure<float, SW>(A, S.rho, S.phi, S.lap[pz][ccol], pm, pz, pp, ccol, rk);
                         acc.J += (double)tw;
@@ -485,6 +534,15 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
                     }
                 }
             }
+        }
+        if constexpr (MASK) {
+            fq1 = fp1;
+            fp0 = fc0;
+            fp1 = fc1;
+            fc0 = fn0;
+            fc1 = fn1;
+            if (fc0 >> 15) gh0 = mk.E[ext_of(yy0 + 2)];
+            if (fc1 >> 15) gh1 = mk.E[ext_of(yy0 + 3)];
         }
         ring_next.advance();
     }
