@@ -281,8 +281,9 @@ __device__ __forceinline__ void grad_rho(const AdjGeo<T> &g, const T *rho, int x
 // density, 1 / density, the equilibrium velocity u_eq = (j + ushift F) / rho (j
 // until the force is known), grad L, phi and dphi/drho = k^2 p0' - 1/3;
 // and, at the rows next to a wall and the columns next to a pressure column
-// only, v = (j + F / 2) / rho and L.
-enum { F_RHO, F_IR, F_UX, F_UY, F_LX, F_LY, F_PHI, F_DPHI, F_VX, F_VY, F_LAP, NFIELD };
+// only, v = (j + F / 2) (1 / rho) and L, and next to a wall v_x as a quotient (the
+// objective's form).
+enum { F_RHO, F_IR, F_UX, F_UY, F_LX, F_LY, F_PHI, F_DPHI, F_VX, F_VY, F_LAP, F_VQ, NFIELD };
 
 // Stored state m of a block: state 0 is the checkpoint, the others follow one
 // another `stride` bytes apart.
@@ -498,6 +499,7 @@ __global__ void __launch_bounds__(TX * TMAX) adj_forces(AdjGeo<T> g, int th, T *
         o[F_VX * n + c] = (X + T(0.5) * FX) * ir;
         o[F_VY * n + c] = (Y + T(0.5) * FY) * ir;
         o[F_LAP * n + c] = lap;
+        o[F_VQ * n + c] = (X + T(0.5) * FX) / r;
     }
 }
 
@@ -732,11 +734,11 @@ __global__ void __launch_bounds__(BLOCK) adj_local(AdjGeo<T> g, int eblocks, con
     // wall objective terms (interior columns; a row may serve both walls on
     // very low channels)
     if (g.walls && (y <= 2 || y >= g.ny - 3)) {
-        const T *rho = fld + F_RHO * N, *vxs = fld + F_VX * N;
+        const T *rho = fld + F_RHO * N;
         for (int side = 0; side < 2; ++side) {
             const int y1 = side ? g.ny - 2 : 1, y2 = side ? g.ny - 3 : 2;
             if (y == y1) {
-                const T v2 = vxs[y2 * g.nx + x];
+                const T v2 = fld[F_VQ * N + y2 * g.nx + x];
                 jbx += g.w_tau * T(3) * g.nu;
                 ax += g.w_tau * T(1.5) * g.nu;
                 rb += -g.w_tau * g.nu / T(3) * v2;
@@ -748,7 +750,7 @@ __global__ void __launch_bounds__(BLOCK) adj_local(AdjGeo<T> g, int eblocks, con
             }
             if (y == y2) {
                 const T r1v = rho[y1 * g.nx + x];
-                const T v2 = vxs[c];
+                const T v2 = fld[F_VX * N + c];
                 jbx += -g.w_tau * g.nu / T(3) * r1v * inv_r;
                 ax += -g.w_tau * g.nu / T(6) * r1v * inv_r;
                 rb += g.w_tau * g.nu / T(3) * r1v * v2 * inv_r;
@@ -1202,8 +1204,8 @@ inline unsigned blocks(long long m) { return (unsigned)((m + TPB - 1) / TPB); }
 
 // Fields of the states of a block are computed for as many states at once as
 // fit this many bytes (at least one): enough to fill the GPU from a small
-// lattice, bounded on a large one.
-constexpr size_t FIELD_BYTES = (size_t)96 << 20;
+// lattice, bounded on a large one. Two such buffers are kept.
+constexpr size_t FIELD_BYTES = (size_t)256 << 20;
 
 } // namespace
 
@@ -1221,11 +1223,17 @@ struct lbm_adjoint {
     int rprec = 64;  // reverse sweep (and objective) arithmetic: 64 or 32
     double dgin = 0, dlin = 0, dgout = 0, dlout = 0;  // d rho_column / d dp
     int64_t held = -1;  // block whose recomputed states blk holds (-1: none)
-    int64_t G = 1;      // states whose fields fld holds
+    int64_t G = 1;      // states whose fields one buffer of fld holds
+    // The backward pass recomputes states and their fields on `prep` while the
+    // reverse chain runs on `chain`, from the other of two field buffers (one
+    // buffer and the caller's stream alone where memory is short).
+    bool overlap = false;
+    cudaStream_t chain = nullptr, prep = nullptr;
+    cudaEvent_t ev_begin = nullptr, ev_end = nullptr, ev_fld[2] = {nullptr, nullptr}, ev_chain[2] = {nullptr, nullptr};
     int sms = 1;
     // device buffers (the reverse sweep's fields and adjoint populations are
     // sized for doubles and hold floats with rprec = 32)
-    double *ckpt = nullptr, *blk = nullptr, *lam0 = nullptr, *lam1 = nullptr, *fld = nullptr;
+    double *ckpt = nullptr, *blk = nullptr, *lam0 = nullptr, *lam1 = nullptr, *fld[2] = {nullptr, nullptr};
     double *Ax = nullptr, *Ay = nullptr, *Jbx = nullptr, *Jby = nullptr, *R = nullptr, *Cw = nullptr;
     double *loads = nullptr, *tw = nullptr, *colp = nullptr, *acc = nullptr, *rho0 = nullptr, *AS = nullptr;
     std::vector<void *> allocs;
@@ -1338,54 +1346,137 @@ int tile_rows(const lbm_adjoint *a, int states)
     return best;
 }
 
-// reverse steps over the n states of block b, last first; lin / lout swap per step
-template <typename T, bool PART>
-lbm_status adj_reverse_block_t(lbm_adjoint *a, int64_t b, int n, double *&lin, double *&lout)
+// A run of states m0 .. m1-1 of block b, walked in reverse from one field buffer.
+struct Run {
+    int64_t b;
+    int m0, m1;
+};
+
+// the fields of a run's states into buffer `buf`, on `st`
+template <typename T>
+lbm_status adj_fields_t(lbm_adjoint *a, const Run &r, int buf, cudaStream_t st)
 {
     const AdjGeo<T> g = geo_as<T>(a->geo);
-    const States st = block_states(a, b);
+    const States states = block_states(a, r.b);
+    const size_t N = (size_t)g.nx * g.ny;
+    const int n = r.m1 - r.m0, fh = tile_rows(a, n);
+    const dim3 ng((unsigned)((N + 127) / 128), n), fg(tiles(g.nx, TX) * tiles(fluid_rows(a->geo), fh), n);
+    T *f = as<T>(a->fld[buf]);
+    if (a->grid.precision == 32) adj_nodes<float, T><<<ng, 128, 0, st>>>(g, states, r.m0, f);
+    else adj_nodes<double, T><<<ng, 128, 0, st>>>(g, states, r.m0, f);
+    adj_forces<T><<<fg, TX * fh, 0, st>>>(g, fh, f);
+    ACK(cudaGetLastError(), "adjoint field kernels");
+    return LBM_OK;
+}
+
+// reverse steps over a run's states, last first; lin / lout swap per step
+template <typename T, bool PART>
+lbm_status adj_chain_t(lbm_adjoint *a, const Run &r, int buf, cudaStream_t st, double *&lin, double *&lout)
+{
+    const AdjGeo<T> g = geo_as<T>(a->geo);
     const size_t N = (size_t)g.nx * g.ny;
     constexpr int LB = sizeof(T) == 8 ? 64 : 128;
     const unsigned eblocks = g.bc_x ? tiles(2 * g.ny, LB) : 0, nblocks = eblocks + (unsigned)((N + LB - 1) / LB);
     const int th = tile_rows(a, 1);
     const unsigned tg = tiles(g.nx, TX) * tiles(fluid_rows(a->geo), th);
-    for (int m1 = n; m1 > 0; m1 -= (int)a->G) {
-        const int m0 = (int)std::max<int64_t>(0, m1 - a->G), fh = tile_rows(a, m1 - m0);
-        const dim3 ng((unsigned)((N + 127) / 128), m1 - m0);
-        const dim3 fg(tiles(g.nx, TX) * tiles(fluid_rows(a->geo), fh), m1 - m0);
-        if (a->grid.precision == 32) adj_nodes<float, T><<<ng, 128, 0, a->stream>>>(g, st, m0, as<T>(a->fld));
-        else adj_nodes<double, T><<<ng, 128, 0, a->stream>>>(g, st, m0, as<T>(a->fld));
-        adj_forces<T><<<fg, TX * fh, 0, a->stream>>>(g, fh, as<T>(a->fld));
-        ACK(cudaGetLastError(), "adjoint field kernels");
-        for (int m = m1 - 1; m >= m0; --m) {
-            const T *f = as<T>(a->fld) + (size_t)(m - m0) * NFIELD * N;
-            T *li = as<T>(lin), *lo = as<T>(lout);
-            ACK(launch_chained(adj_local<T, PART, LB>, dim3(nblocks), dim3(LB), a->stream, g, (int)eblocks, li, f, lo,
-                               as<T>(a->Ax), as<T>(a->Ay), as<T>(a->Jbx), as<T>(a->Jby), as<T>(a->R), as<T>(a->Cw),
-                               a->AS),
-                "adjoint local kernel");
-            auto finish = adj_finish<T, PART>;
-            if constexpr (BY_TERMS<T>) {
-                if (g.walls && g.bc_x) finish = adj_finish_terms<PART>;
-            }
-            ACK(launch_chained(finish, dim3(tg), dim3(TX * th), a->stream, g, th, f, as<T>(a->Ax), as<T>(a->Ay),
-                               as<T>(a->Jbx), as<T>(a->Jby), as<T>(a->R), as<T>(a->Cw), lo, a->colp),
-                "adjoint finish kernel");
-            std::swap(lin, lout);
+    for (int m = r.m1 - 1; m >= r.m0; --m) {
+        const T *f = as<T>(a->fld[buf]) + (size_t)(m - r.m0) * NFIELD * N;
+        T *li = as<T>(lin), *lo = as<T>(lout);
+        ACK(launch_chained(adj_local<T, PART, LB>, dim3(nblocks), dim3(LB), st, g, (int)eblocks, li, f, lo,
+                           as<T>(a->Ax), as<T>(a->Ay), as<T>(a->Jbx), as<T>(a->Jby), as<T>(a->R), as<T>(a->Cw), a->AS),
+            "adjoint local kernel");
+        auto finish = adj_finish<T, PART>;
+        if constexpr (BY_TERMS<T>) {
+            if (g.walls && g.bc_x) finish = adj_finish_terms<PART>;
         }
+        ACK(launch_chained(finish, dim3(tg), dim3(TX * th), st, g, th, f, as<T>(a->Ax), as<T>(a->Ay), as<T>(a->Jbx),
+                           as<T>(a->Jby), as<T>(a->R), as<T>(a->Cw), lo, a->colp),
+            "adjoint finish kernel");
+        std::swap(lin, lout);
     }
     return LBM_OK;
 }
 
-lbm_status adj_reverse_block(lbm_adjoint *a, int64_t b, int n, double *&lin, double *&lout)
+lbm_status adj_run_fields(lbm_adjoint *a, const Run &r, int buf, cudaStream_t st)
+{
+    return a->rprec == 32 ? adj_fields_t<float>(a, r, buf, st) : adj_fields_t<double>(a, r, buf, st);
+}
+lbm_status adj_run_chain(lbm_adjoint *a, const Run &r, int buf, cudaStream_t st, double *&lin, double *&lout)
 {
     // without MRT and at tau = 1 the relaxation leaves nothing of f*-bar
     const bool part = a->geo.mrt || a->geo.inv_tau != 1.0;
     if (a->rprec == 32)
-        return part ? adj_reverse_block_t<float, true>(a, b, n, lin, lout)
-                    : adj_reverse_block_t<float, false>(a, b, n, lin, lout);
-    return part ? adj_reverse_block_t<double, true>(a, b, n, lin, lout)
-                : adj_reverse_block_t<double, false>(a, b, n, lin, lout);
+        return part ? adj_chain_t<float, true>(a, r, buf, st, lin, lout)
+                    : adj_chain_t<float, false>(a, r, buf, st, lin, lout);
+    return part ? adj_chain_t<double, true>(a, r, buf, st, lin, lout)
+                : adj_chain_t<double, false>(a, r, buf, st, lin, lout);
+}
+
+// The whole reverse sweep: block by block, last first, each in runs of at most G
+// states. Preparing run i + 1 (recomputing its block's states first, where it
+// opens one: by then the fields of every state in their storage are taken)
+// does not depend on the adjoint, so it overlaps the chain of run i, whose two
+// short kernels per step leave half of the FP64 pipe idle (512 x 128, 200 steps
+// forward and back: 14.1 ms one after the other, 11.4 overlapped; 1024 x 256
+// with an FP32 reverse, 100 steps: 6.2 and 5.7). Run i's fields lie in buffer
+// i & 1, free again once chain i - 2 is through.
+lbm_status adj_sweep(lbm_adjoint *a, double *&lin, double *&lout)
+{
+    std::vector<Run> runs;
+    for (int64_t b = a->nblocks - 1; b >= 0; --b) {
+        const int n = (int)(std::min(a->nsteps, (b + 1) * a->K) - b * a->K);
+        const int parts = (int)((n + a->G - 1) / a->G), len = (n + parts - 1) / parts;
+        for (int m1 = n; m1 > 0; m1 -= len) runs.push_back(Run{b, std::max(0, m1 - len), m1});
+    }
+    const bool ov = a->overlap;
+    const cudaStream_t prep = ov ? a->prep : a->stream, chain = ov ? a->chain : a->stream;
+    lbm_status s;
+    auto prepare = [&](size_t i) -> lbm_status {
+        const Run &r = runs[i];
+        if (a->held != r.b) {
+            a->held = -1;
+            const int64_t n0 = r.b * a->K, n1 = std::min(a->nsteps, n0 + a->K);
+            for (int64_t t = n0; t + 1 < n1; ++t)
+                ACK(lbm_ctx_step_between(a->ctx, state_of(a, t), state_of(a, t + 1), prep), "recompute step");
+            a->held = r.b;
+        }
+        const int buf = ov ? (int)(i & 1) : 0;
+        if (ov && i >= 2) ACK(cudaStreamWaitEvent(prep, a->ev_chain[buf], 0), "adjoint event");
+        if ((s = adj_run_fields(a, r, buf, prep)) != LBM_OK) return s;
+        if (ov) ACK(cudaEventRecord(a->ev_fld[buf], prep), "adjoint event");
+        return LBM_OK;
+    };
+    if (ov) {
+        ACK(cudaEventRecord(a->ev_begin, a->stream), "adjoint event");
+        ACK(cudaStreamWaitEvent(prep, a->ev_begin, 0), "adjoint event");
+        ACK(cudaStreamWaitEvent(chain, a->ev_begin, 0), "adjoint event");
+        if ((s = prepare(0)) != LBM_OK) return s;
+    }
+    for (size_t i = 0; i < runs.size(); ++i) {
+        const int buf = ov ? (int)(i & 1) : 0;
+        if (!ov) {
+            if ((s = prepare(i)) != LBM_OK) return s;
+        } else {
+            if (i + 1 < runs.size() && (s = prepare(i + 1)) != LBM_OK) return s;
+            ACK(cudaStreamWaitEvent(chain, a->ev_fld[buf], 0), "adjoint event");
+        }
+        if ((s = adj_run_chain(a, runs[i], buf, chain, lin, lout)) != LBM_OK) return s;
+        if (ov) ACK(cudaEventRecord(a->ev_chain[buf], chain), "adjoint event");
+    }
+    if (ov) {  // every event of `prep` was waited for on `chain`
+        ACK(cudaEventRecord(a->ev_end, chain), "adjoint event");
+        ACK(cudaStreamWaitEvent(a->stream, a->ev_end, 0), "adjoint event");
+    }
+    return LBM_OK;
+}
+
+// Work left on the internal streams by a call that failed half way is finished
+// before anything new is enqueued.
+cudaError_t adj_drain(lbm_adjoint *a)
+{
+    if (!a->overlap) return cudaSuccess;
+    cudaError_t e = cudaStreamSynchronize(a->prep);
+    return e == cudaSuccess ? cudaStreamSynchronize(a->chain) : e;
 }
 
 // the error word of the forward context's steps, read with the results
@@ -1395,6 +1486,33 @@ lbm_status step_errors(lbm_adjoint *a, int word, const char *what)
     const lbm_status s = word & 1 ? LBM_ERR_NAN : LBM_ERR_TIMEOUT;
     a->err = std::string(what) + ": " + lbm_status_string(s);
     return s;
+}
+
+// the sweep's internal streams and events; false (nothing kept) on failure.
+// The chain, whose kernels are short and wait for one another, goes first
+// where both have blocks to place.
+void adj_streams_free(lbm_adjoint *a)
+{
+    for (cudaEvent_t *e : {&a->ev_begin, &a->ev_end, &a->ev_fld[0], &a->ev_fld[1], &a->ev_chain[0], &a->ev_chain[1]}) {
+        if (*e) cudaEventDestroy(*e);
+        *e = nullptr;
+    }
+    for (cudaStream_t *st : {&a->chain, &a->prep}) {
+        if (*st) cudaStreamDestroy(*st);
+        *st = nullptr;
+    }
+}
+bool adj_streams(lbm_adjoint *a)
+{
+    int least = 0, greatest = 0;
+    cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&a->chain, cudaStreamNonBlocking, greatest);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&a->prep, cudaStreamNonBlocking, least);
+    for (cudaEvent_t *ev : {&a->ev_begin, &a->ev_end, &a->ev_fld[0], &a->ev_fld[1], &a->ev_chain[0], &a->ev_chain[1]})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) return true;
+    adj_streams_free(a);
+    return false;
 }
 
 lbm_status ctx_status(lbm_adjoint *a, lbm_status s, const char *what)
@@ -1510,15 +1628,28 @@ lbm_status lbm_adjoint_init(const lbm_grid *grid, const lbm_eos *eos, double tau
         {&a->AS, 2 * n}};
     for (auto &b : bufs)
         if (s == LBM_OK) s = adj_alloc(a, b.p, b.count);
-    // the fields of one state at a time where memory is short
-    const size_t F = NFIELD * n + 4 * (size_t)grid->nx;
-    if (s == LBM_OK && a->G > 1 && adj_alloc(a, &a->fld, F * a->G) != LBM_OK) {
-        cudaGetLastError();
-        a->G = 1;
+    // Two field buffers and the overlapped sweep, or, where memory is short, the
+    // fields of one state at a time on the caller's stream. The runs of a block
+    // are of even length.
+    const int64_t parts = (a->K + a->G - 1) / a->G;
+    a->G = (a->K + parts - 1) / parts;
+    const size_t F = NFIELD * n;
+    if (s == LBM_OK) {
+        double *two = nullptr;
+        if (adj_alloc(a, &two, 2 * F * a->G + 4 * (size_t)grid->nx * a->G) == LBM_OK && adj_streams(a)) {
+            a->fld[0] = two;
+            a->fld[1] = two + F * a->G;
+            a->loads = two + 2 * F * a->G;
+            a->overlap = true;
+        } else {
+            cudaGetLastError();
+            a->err.clear();
+            a->G = 1;
+            s = adj_alloc(a, &a->fld[0], F + 4 * (size_t)grid->nx);
+            a->loads = a->fld[0] ? a->fld[0] + F : nullptr;
+        }
     }
-    if (s == LBM_OK && !a->fld) s = adj_alloc(a, &a->fld, F);
     if (s != LBM_OK) { lbm_adjoint_free(a); return s; }
-    a->loads = a->fld + NFIELD * n * a->G;
     // slots that no population reaches and padding columns are never read as
     // lattice nodes; they start at zero once
     if (cudaMemsetAsync(a->ckpt, 0, SD * 8 * a->nblocks, a->stream) != cudaSuccess ||
@@ -1538,6 +1669,7 @@ lbm_status lbm_adjoint_forward(lbm_adjoint *a, const lbm_drive *drive, const dou
 {
     if (!a || !rho0 || !J) return LBM_ERR_ARG;
     a->forward_done = false;
+    ACK(adj_drain(a), "adjoint streams");
     lbm_status s = adj_setup_drive(a, drive);
     if (s != LBM_OK) return s;
     const long long n = (long long)a->grid.nx * a->grid.ny;
@@ -1556,7 +1688,7 @@ lbm_status lbm_adjoint_forward(lbm_adjoint *a, const lbm_drive *drive, const dou
     // of a block's states are taken together once they are all there.
     for (int64_t t = 0; t < a->nsteps; ++t) {
         const bool last = t + 1 == a->nsteps;
-        if (!last) ACK(lbm_ctx_step_between(a->ctx, state_of(a, t), state_of(a, t + 1)), "forward step");
+        if (!last) ACK(lbm_ctx_step_between(a->ctx, state_of(a, t), state_of(a, t + 1), a->stream), "forward step");
         // the step that ends a block writes the next checkpoint, not the block
         if ((last || (t + 1) % a->K == 0) && (s = adj_objective(a, t / a->K, (int)(t % a->K) + 1)) != LBM_OK) return s;
     }
@@ -1581,6 +1713,7 @@ lbm_status lbm_adjoint_backward(lbm_adjoint *a, double w_tau, double w_p, double
     if (!a || !grad_rho0 || !grad_drive) return LBM_ERR_ARG;
     if (!a->forward_done) { a->err = "backward before forward"; return LBM_ERR_STATE; }
     if (!std::isfinite(w_tau) || !std::isfinite(w_p)) return LBM_ERR_ARG;
+    ACK(adj_drain(a), "adjoint streams");
     a->geo.w_tau = w_tau;
     a->geo.w_p = w_p;
     const long long n = (long long)a->grid.nx * a->grid.ny;
@@ -1593,16 +1726,7 @@ lbm_status lbm_adjoint_backward(lbm_adjoint *a, double w_tau, double w_p, double
     ACK(cudaMemsetAsync(a->colp, 0, 4 * (size_t)a->grid.ny * sizeof(double), a->stream), "adjoint memset");
     double *lin = a->lam1, *lout = a->lam0;
     lbm_status s;
-    for (int64_t b = a->nblocks - 1; b >= 0; --b) {
-        const int64_t n0 = b * a->K, n1 = std::min(a->nsteps, n0 + a->K);
-        if (a->held != b) {
-            a->held = -1;
-            for (int64_t t = n0; t + 1 < n1; ++t)
-                ACK(lbm_ctx_step_between(a->ctx, state_of(a, t), state_of(a, t + 1)), "recompute step");
-            a->held = b;
-        }
-        if ((s = adj_reverse_block(a, b, (int)(n1 - n0), lin, lout)) != LBM_OK) return s;
-    }
+    if ((s = adj_sweep(a, lin, lout)) != LBM_OK) return s;
     // per-node and per-row sums over the steps, reduced once
     adj_reduce_col<<<1, RED_THREADS, 0, a->stream>>>(a->colp, a->grid.ny, a->acc + 2);
     adj_reduce<<<1, RED_THREADS, 0, a->stream>>>(a->AS, n, n, 2, a->acc + 6);
@@ -1658,7 +1782,9 @@ const char *lbm_adjoint_last_error(const lbm_adjoint *a) { return a ? a->err.c_s
 void lbm_adjoint_free(lbm_adjoint *a)
 {
     if (!a) return;
+    adj_drain(a);
     if (a->ctx) lbm_free(a->ctx);
+    adj_streams_free(a);
     for (void *p : a->allocs) cudaFree(p);
     delete a;
 }

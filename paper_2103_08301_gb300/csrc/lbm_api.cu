@@ -721,10 +721,15 @@ cudaError_t step_between(lbm_ctx *ctx, const void *fin, void *fout)
 }
 }  // namespace
 
-cudaError_t lbm_ctx_step_between(lbm_ctx *ctx, const void *fin, void *fout)
+cudaError_t lbm_ctx_step_between(lbm_ctx *ctx, const void *fin, void *fout, cudaStream_t stream)
 {
     if (ctx->inplace || ctx->mask || ctx->tile) return cudaErrorNotSupported;
-    return ctx->grid.precision == 64 ? step_between<double>(ctx, fin, fout) : step_between<float>(ctx, fin, fout);
+    const cudaStream_t own = ctx->stream;
+    ctx->stream = stream;
+    const cudaError_t e =
+        ctx->grid.precision == 64 ? step_between<double>(ctx, fin, fout) : step_between<float>(ctx, fin, fout);
+    ctx->stream = own;
+    return e;
 }
 
 int *lbm_ctx_error_word(lbm_ctx *ctx) { return (int *)(ctx->ws + ctx->L.err); }

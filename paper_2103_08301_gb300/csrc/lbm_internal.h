@@ -82,11 +82,11 @@ inline int strip_width(int nx, int w_max, bool bc_x)
 bool lbm_encode_population_map(CUtensorMap *map, void *base, int pitch, int ny);
 // One step of a context between two states outside it, each in the context's
 // own layout (rows of nine planes, plane pitch pitch_of(nx), 9 * pitch * ny
-// values, 256-byte aligned), on the context's stream; slots that no population
+// values, 256-byte aligned), on `stream`; slots that no population
 // reaches keep their contents in `fout`. The context's own state and step
 // counter are untouched; bad densities are flagged in its error word (device),
 // lbm_ctx_error_word. Two-array contexts without a wall mask. lbm_api.cu.
-cudaError_t lbm_ctx_step_between(lbm_ctx *ctx, const void *fin, void *fout);
+cudaError_t lbm_ctx_step_between(lbm_ctx *ctx, const void *fin, void *fout, cudaStream_t stream);
 int *lbm_ctx_error_word(lbm_ctx *ctx);
 
 namespace lbm {
