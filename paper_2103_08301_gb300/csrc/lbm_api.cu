@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <new>
 
 #include "lbm.h"
@@ -702,6 +703,25 @@ struct CkptHeader {
 
 } // namespace
 
+namespace {
+// A checkpoint's per-CTA partials for a plan of n CTAs: those of a plan with
+// more CTAs are folded into the first n, so that the totals stay.
+template <typename real>
+void fold_partials(double *mass, double *J, real *ext, int n)
+{
+    for (int c = n; c < lbm::MAX_CTAS; ++c) {
+        mass[c % n] += mass[c];
+        J[c % n] += J[c];
+        mass[c] = J[c] = 0.0;
+        real *to = ext + 4 * (c % n), *from = ext + 4 * c;
+        for (int k = 0; k < 4; ++k) {
+            to[k] = k & 1 ? std::max(to[k], from[k]) : std::min(to[k], from[k]);
+            from[k] = k & 1 ? -INFINITY : INFINITY;
+        }
+    }
+}
+} // namespace
+
 bool lbm_encode_population_map(CUtensorMap *map, void *base, int pitch, int ny)
 {
     return encode_population_map(map, base, pitch, ny);
@@ -1152,22 +1172,25 @@ lbm_status lbm_restore(lbm_ctx *ctx, const void *host_buf, size_t bytes)
     const size_t sz = ctx->grid.precision == 64 ? 8 : 4;
     const int narr = ctx->inplace ? 1 : 2;
     const unsigned char *p = (const unsigned char *)host_buf + sizeof h;
+    const size_t nparts = (size_t)lbm::MAX_CTAS * (16 + 4 * sz);
+    std::unique_ptr<unsigned char[]> part(new (std::nothrow) unsigned char[nparts]);
+    if (!part) return LBM_ERR_OOM;
     CK(cudaMemcpyAsync(ctx->ws + ctx->L.f0, p, narr * ctx->L.pops, cudaMemcpyHostToDevice, ctx->stream), "restore");
     p += narr * ctx->L.pops;
-    CK(cudaMemcpyAsync(ctx->ws + ctx->L.mass, p, lbm::MAX_CTAS * 8, cudaMemcpyHostToDevice, ctx->stream), "restore");
-    p += lbm::MAX_CTAS * 8;
-    CK(cudaMemcpyAsync(ctx->ws + ctx->L.J, p, lbm::MAX_CTAS * 8, cudaMemcpyHostToDevice, ctx->stream), "restore");
-    p += lbm::MAX_CTAS * 8;
-    CK(cudaMemcpyAsync(ctx->ws + ctx->L.ext, p, lbm::MAX_CTAS * 4 * sz, cudaMemcpyHostToDevice, ctx->stream), "restore");
-    p += lbm::MAX_CTAS * 4 * sz;
+    std::memcpy(part.get(), p, nparts);
+    unsigned char *mass = part.get(), *J = mass + lbm::MAX_CTAS * 8, *ext = J + lbm::MAX_CTAS * 8;
+    if (ctx->grid.precision == 64) fold_partials((double *)mass, (double *)J, (double *)ext, diag_ctas(ctx));
+    else fold_partials((double *)mass, (double *)J, (float *)ext, diag_ctas(ctx));
+    p += nparts;
+    CK(cudaMemcpyAsync(ctx->ws + ctx->L.mass, mass, lbm::MAX_CTAS * 8, cudaMemcpyHostToDevice, ctx->stream), "restore");
+    CK(cudaMemcpyAsync(ctx->ws + ctx->L.J, J, lbm::MAX_CTAS * 8, cudaMemcpyHostToDevice, ctx->stream), "restore");
+    CK(cudaMemcpyAsync(ctx->ws + ctx->L.ext, ext, lbm::MAX_CTAS * 4 * sz, cudaMemcpyHostToDevice, ctx->stream), "restore");
     CK(cudaMemcpyAsync(ctx->ws + ctx->L.err, p, sizeof(int), cudaMemcpyHostToDevice, ctx->stream), "restore");
     CK(cudaStreamSynchronize(ctx->stream), "restore sync");
     ctx->step = h.step;
     ctx->cur = h.cur;
     ctx->aa_odd = false;
     ctx->err_pending = false;
-    // Per-CTA accumulators only line up with the same launch geometry; with
-    // another CTA count they stay valid as totals but the summation order changes.
     ctx->nctas = std::max(ctx->nctas, 1);
     return LBM_OK;
 }
@@ -1249,10 +1272,11 @@ lbm_status lbm_set_option(lbm_ctx *ctx, lbm_option opt, int64_t value)
     }
     // Re-plan; per-CTA accumulators are folded into the new partition only
     // through their totals, so reset them to keep the reduction exact.
-    int old = ctx->nctas;
+    const int old = ctx->nctas;
+    const bool was_general = ctx->mask != nullptr;
     lbm_status s = plan_launch(ctx);
     if (s == LBM_OK) s = plan_geometry(ctx);
-    if (s == LBM_OK && old != ctx->nctas) {
+    if (s == LBM_OK && (old != ctx->nctas || was_general != (ctx->mask != nullptr))) {
         if (ctx->grid.precision == 64) reset_acc<double>(ctx); else reset_acc<float>(ctx);
     }
     return s;
