@@ -116,6 +116,9 @@ struct lbm_ctx {
     // in-place steps since it last held the natural one)
     bool inplace = false, aa_odd = false;
     lbm::AAPlan aa{};
+    // its FP32 step by row pairs in place (long segments): strip plan and maps
+    struct { bool on; int W, nstrips, nctas, band; long long units; } aas{};
+    CUtensorMap tmap_aa[3];  // boxes of AA_SP columns by 9, 1 and 2 planes
     int64_t step = 0;
     int W = STRIP, nstrips = 0, yf0 = 0, nyf = 0;
     int W_opt = 0;  // LBM_OPT_STRIP (0: widest)
@@ -322,13 +325,14 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
 // The 2-D view of one FP32 population buffer that the row-pair stage reads:
 // x = column (pitch wide, stride 4 pitch bytes per y), y = 9 * row + plane;
 // boxes of R2_SP columns by 9 planes (one stencil row), zero fill outside.
-bool encode_population_map(CUtensorMap *map, void *base, int pitch, int ny, int box_cols = lbm::R2_SP)
+bool encode_population_map(CUtensorMap *map, void *base, int pitch, int ny, int box_cols = lbm::R2_SP,
+                           unsigned box_planes = 9)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc || pitch % 4 != 0) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)pitch, (cuuint64_t)9 * (cuuint64_t)ny};
     const cuuint64_t strides[1] = {(cuuint64_t)pitch * sizeof(float)};
-    const cuuint32_t box[2] = {(cuuint32_t)box_cols, 9u};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, box_planes};
     const cuuint32_t elem[2] = {1u, 1u};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -553,6 +557,20 @@ template <typename real>
 lbm_status one_step(lbm_ctx *ctx)
 {
     lbm::KArgs<real> A = make_args<real>(ctx);
+    if (ctx->inplace && ctx->aas.on) {
+        lbm::KArgs<float> B = make_args<float>(ctx);
+        B.W = ctx->aas.W;
+        B.nstrips = ctx->aas.nstrips;
+        B.units = ctx->aas.units;
+        B.nctas = ctx->aas.nctas;
+        B.band = ctx->aas.band;
+        cudaError_t e = lbm::aa_strips_step(B, (float *)(ctx->ws + ctx->L.f0), (float *)(ctx->ws + ctx->L.rho), ctx->tmap_aa,
+                                            ctx->grid.walls, ctx->aa_odd, ctx->big, ctx->sms, ctx->stream);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "in-place step launch");
+        ctx->aa_odd = !ctx->aa_odd;
+        ctx->step += 1;
+        return LBM_OK;
+    }
     if (ctx->inplace) {
         cudaError_t e = lbm::aa_step<real>(A, (real *)(ctx->ws + ctx->L.f0), (real *)(ctx->ws + ctx->L.rho),
                                            (real *)(ctx->ws + ctx->L.side), ctx->grid.walls, ctx->grid.bc_x,
@@ -618,7 +636,10 @@ lbm_status aa_natural(lbm_ctx *ctx)
 }
 
 // CTAs whose diagnostic slots hold the step's partials
-int diag_ctas(const lbm_ctx *ctx) { return ctx->inplace ? ctx->aa.nctas : ctx->nctas; }
+int diag_ctas(const lbm_ctx *ctx)
+{
+    return !ctx->inplace ? ctx->nctas : (ctx->aas.on ? ctx->aas.nctas : ctx->aa.nctas);
+}
 
 template <typename real>
 lbm_status do_fields(lbm_ctx *ctx, void *rho, void *ux, void *uy, void *tw, void *pw)
@@ -755,6 +776,38 @@ cudaError_t lbm_ctx_step_between(lbm_ctx *ctx, const void *fin, void *fout, cuda
 int *lbm_ctx_error_word(lbm_ctx *ctx) { return (int *)(ctx->ws + ctx->L.err); }
 
 namespace {
+
+// In-place FP32 contexts between pressure columns whose row-pair plan gives CTAs
+// AA_ROWS_MIN rows or more: the step by row pairs in place. A segment's first rows
+// are filled from the density plane, so short segments keep the tiles, whose cost
+// does not depend on segments (us per step, tiles against strips: 8192 x 1024,
+// 94 rows, 218 and 181; 8192 x 768, 70 rows, 166 and 141; 4096 x 1024, 47 rows,
+// 113 and 109; 4096 x 512, 24 rows, 53 and 65).
+constexpr long long AA_ROWS_MIN = 48;
+lbm_status plan_inplace_strips(lbm_ctx *ctx)
+{
+    auto &s = ctx->aas;
+    s = {};
+    const lbm_grid &g = ctx->grid;
+    if (g.precision != 32 || !g.bc_x || ctx->pitch % 4 != 0) return LBM_OK;
+    s.W = lbm::strip_width(g.nx, lbm::AA_W, true);
+    if (s.W % 4 != 0) return LBM_OK;
+    s.nstrips = (g.nx + s.W - 1) / s.W;
+    s.units = (long long)s.nstrips * ctx->nyf;
+    int per_sm = 0;
+    cudaError_t e = lbm::aa_strips_plan(g.walls, ctx->big, &per_sm);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "in-place strip plan");
+    s.nctas = (int)std::max<long long>(1, std::min<long long>({(long long)ctx->sms * std::max(1, per_sm), s.units / 2,
+                                                               (long long)lbm::MAX_CTAS}));
+    if (s.units < AA_ROWS_MIN * s.nctas) return LBM_OK;
+    s.band = band_rows(ctx->nyf, s.nstrips, s.nctas, g.walls);
+    static const unsigned planes[3] = {9, 1, 2};
+    for (int k = 0; k < 3; ++k)
+        if (!encode_population_map(&ctx->tmap_aa[k], ctx->ws + ctx->L.f0, ctx->pitch, g.ny, lbm::AA_SP, planes[k]))
+            return LBM_OK;
+    s.on = true;
+    return LBM_OK;
+}
 
 // (Re)selects the general-geometry path: kept when the caller's mask adds
 // solid nodes to the wall rows or LBM_OPT_GENERAL forces it; the diagnostic
@@ -914,6 +967,11 @@ lbm_status init_ctx(const lbm_grid *grid, const lbm_eos *eos, double tau, const 
             lbm_free(ctx);
             return s;
         }
+    }
+
+    if (inplace) {
+        st = plan_inplace_strips(ctx);
+        if (st != LBM_OK) { lbm_free(ctx); return st; }
     }
 
     // Initial state f = f_eq(rho0, 0) in both arrays (in-place contexts: the
@@ -1286,6 +1344,13 @@ lbm_status lbm_launch_info(const lbm_ctx *ctx, int64_t *ctas, int64_t *threads, 
                            int64_t *staged)
 {
     if (!ctx) return LBM_ERR_ARG;
+    if (ctx->inplace && ctx->aas.on) {
+        if (ctas) *ctas = ctx->aas.nctas;
+        if (threads) *threads = lbm::R2_BLOCK;
+        if (units) *units = ctx->aas.units;
+        if (staged) *staged = 1;
+        return LBM_OK;
+    }
     if (ctx->inplace) {
         // CTAs striding over the 32 x 8 tiles (FP32: two rows per thread)
         if (ctas) *ctas = ctx->aa.nctas;

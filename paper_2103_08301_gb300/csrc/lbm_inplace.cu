@@ -27,7 +27,9 @@
 //
 // Traffic per node and step (FP32): 36 B read and 4 B written by the density
 // pass, 36 B read, 36 B written and 4 B of densities read by the step, 116 B
-// against the two-array step's 72 B; storage 40 B against 72 B.
+// against the two-array step's 72 B; storage 40 B against 72 B. Large FP32
+// channels between pressure columns step by row pairs instead, with densities
+// from the plane for the halo only (aa_step_kernel_rows2): about 76 B.
 
 #include <cuda_runtime.h>
 
@@ -721,6 +723,118 @@ __global__ void __launch_bounds__(AA2_THREADS, LBM_AA2_MIN_BLOCKS)
 }
 
 // ---------------------------------------------------------------------------
+// Long channels (FP32, pressure columns, row-pair plan of long segments): the
+// row-pair kernel marches in place (lbm_rows2.cuh, AA). Only the densities that a
+// segment reads outside itself come from the plane: four columns around every
+// strip boundary and four rows around every cut, about a twentieth of the
+// lattice, instead of a density pass over all of it. 16384 x 2048: 0.837 ms a step
+// by tiles (density pass 0.211 of it), 0.668 by row pairs; the two-array step, with
+// 40 bytes a node less to move than the tiles and 4 less than this, 0.472.
+// ---------------------------------------------------------------------------
+
+template <bool ODD, typename IX>
+__device__ __forceinline__ float aa_sum(const float *F, int x, int y, int ny, int P, bool walls)
+{
+    float f[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        if (ODD) {
+            const int sy = walls ? y - ey_(i) : wrap1(y - ey_(i), ny);
+            f[i] = F[aa_slot<IX>(x - ex_(i), sy, opp_(i), P)];
+        } else {
+            f[i] = F[aa_slot<IX>(x, y, i, P)];
+        }
+    }
+    const float s = add_(add_(add_(f[0], f[1]), add_(f[2], f[3])), add_(add_(f[4], f[5]), add_(f[6], f[7])));
+    return add_(s, f[8]);
+}
+
+// Block c < A.nctas: the rows next to CTA c's segments (columns 1 .. nx-2 of the
+// strip and two beyond); the other blocks: columns x0-2 .. x0+1 of every strip
+// boundary x0, all fluid rows.
+template <bool WALLS, bool ODD, typename IX>
+__global__ void __launch_bounds__(128) aa_halo_kernel(const KArgs<float> A, const float *F, float *rho, int cblocks)
+{
+    const int nx = A.nx, ny = A.ny, P = A.pitch;
+    if ((int)blockIdx.x < A.nctas) {
+        long long u = cut_units<WALLS>(A, blockIdx.x);
+        const long long u1 = cut_units<WALLS>(A, blockIdx.x + 1);
+        while (u < u1) {
+            int s, ya;
+            long long run_end;
+            unit_run(A, u, s, ya, run_end);
+            const long long ue = min(u1, run_end);
+            const int yb = ya + (int)(ue - u);
+            u = ue;
+            const int xl = max(1, s * A.W - 2), xr = min(nx - 2, min(s * A.W + A.W, nx) + 1);
+            const int w = xr - xl + 1;
+            for (int k = threadIdx.x; k < 4 * w; k += 128) {
+                const int q = k / w, x = xl + k - q * w, yy = q < 2 ? ya - 2 + q : yb + q - 2;
+                bool mir;
+                const int y = map_row<WALLS>(yy, ny, mir);
+                if (!mir) rho[(IX)y * P + x] = aa_sum<ODD, IX>(F, x, y, ny, P, WALLS);
+            }
+        }
+        return;
+    }
+    const long long n = (long long)(A.nstrips - 1) * 4 * A.nyf;
+    for (long long k = (blockIdx.x - A.nctas) * 128ll + threadIdx.x; k < n; k += cblocks * 128ll) {
+        const int per_row = (A.nstrips - 1) * 4, yl = (int)(k / per_row), c = (int)(k - (long long)yl * per_row);
+        const int x = (c / 4 + 1) * A.W - 2 + (c & 3), y = A.yf0 + yl;
+        if (x <= nx - 2) rho[(IX)y * P + x] = aa_sum<ODD, IX>(F, x, y, ny, P, WALLS);
+    }
+}
+
+template <bool WALLS, int AA, typename IX>
+__global__ void __launch_bounds__(R2_BLOCK, LBM_R2_MIN_BLOCKS)
+    aa_step_kernel_rows2(const KArgs<float> A, const __grid_constant__ CUtensorMap m9, const __grid_constant__ CUtensorMap m1,
+                         const __grid_constant__ CUtensorMap m2, const float *rho)
+{
+    extern __shared__ __align__(128) unsigned char dsm[];
+    float *const stages = reinterpret_cast<float *>(dsm);
+    uint64_t *const bars = reinterpret_cast<uint64_t *>(dsm + (size_t)R2_SLOTS * 18 * AA_SP * sizeof(float));
+    __shared__ SmemR2 S;
+    const int tid = threadIdx.x;
+    const int cta = A.reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+    long long u = cut_units<WALLS>(A, cta);
+    const long long u1 = cut_units<WALLS>(A, cta + 1);
+    const Geom<float> G{A.fin, A.fout, A.nx, A.ny, A.W, A.pitch, A.rho_in_g, A.rho_in_l, A.rho_out_g, A.rho_out_l};
+    Acc<float, 1> acc;
+    acc.reset();
+    RingPos2 ring_next;
+    bool lost = false;
+    if (tid == 0) {
+        for (int st = 0; st < R2_SLOTS; ++st) mbar_init(&bars[st], 1);
+        mbar_init_fence();
+    }
+    __syncthreads();
+    while (u < u1) {
+        int s, ya;
+        long long run_end;
+        unit_run(A, u, s, ya, run_end);
+        const long long ue = min(u1, run_end);
+        const int yb = ya + (int)(ue - u);
+        u = ue;
+        run_segment_r2<WALLS, true, true, false, IX, 1, false, false, AA>(A, G, s, ya, yb, S, stages, bars, ring_next, &m9,
+                                                                          acc, lost, false, nullptr, MaskR2{},
+                                                                          AAStrips{rho, &m1, &m2});
+    }
+    if (lost) atomicOr(A.err, 2);
+    double m, j;
+    float e[4];
+    bool anybad;
+    cta_reduce<float, R2_BLOCK, 1>(acc, S, m, j, e, anybad);
+    if (tid == 0) {
+        A.mass_part[cta] = m;
+        A.J_acc[cta] += j;
+        float *ex = A.ext + 4 * cta;
+        ex[0] = fmin(ex[0], e[0]); ex[1] = fmax(ex[1], e[1]);
+        ex[2] = fmin(ex[2], e[2]); ex[3] = fmax(ex[3], e[3]);
+        if (anybad) atomicOr(A.err, 1);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Host side: kernel selection, the tile plan and the launches.
 // ---------------------------------------------------------------------------
 namespace {
@@ -794,6 +908,56 @@ template <typename real>
 constexpr int step_threads() { return sizeof(real) == 4 ? AA2_THREADS : AA_THREADS; }
 
 }  // namespace
+
+namespace {
+constexpr size_t AA_STRIP_SMEM = (size_t)R2_SLOTS * 18 * AA_SP * sizeof(float) + R2_SLOTS * sizeof(uint64_t);
+template <typename IX>
+void *aa_rows2_fn(bool walls, bool odd)
+{
+    if (walls) return odd ? (void *)aa_step_kernel_rows2<true, 2, IX> : (void *)aa_step_kernel_rows2<true, 1, IX>;
+    return odd ? (void *)aa_step_kernel_rows2<false, 2, IX> : (void *)aa_step_kernel_rows2<false, 1, IX>;
+}
+template <typename IX>
+void *aa_halo_fn(bool walls, bool odd)
+{
+    if (walls) return odd ? (void *)aa_halo_kernel<true, true, IX> : (void *)aa_halo_kernel<true, false, IX>;
+    return odd ? (void *)aa_halo_kernel<false, true, IX> : (void *)aa_halo_kernel<false, false, IX>;
+}
+}  // namespace
+
+cudaError_t aa_strips_plan(bool walls, bool big, int *ctas_per_sm)
+{
+    *ctas_per_sm = 1 << 20;
+    for (bool odd : {false, true}) {
+        void *fn = big ? aa_rows2_fn<long long>(walls, odd) : aa_rows2_fn<int>(walls, odd);
+        int occ = 0;
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AA_STRIP_SMEM);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, R2_BLOCK, AA_STRIP_SMEM);
+        if (e != cudaSuccess) return e;
+        *ctas_per_sm = std::min(*ctas_per_sm, occ);
+    }
+    return cudaSuccess;
+}
+
+cudaError_t aa_strips_step(const KArgs<float> &A, float *F, float *rho, const CUtensorMap *maps, bool walls, bool odd,
+                           bool big, int sms, cudaStream_t st)
+{
+    const float *Fc = F, *rc = rho;
+    const long long n = (long long)(A.nstrips - 1) * 4 * A.nyf;
+    int cblocks = (int)std::max<long long>(1, std::min<long long>((n + 127) / 128, (long long)sms * 16));
+    void *hargs[] = {(void *)&A, (void *)&Fc, (void *)&rho, (void *)&cblocks};
+    cudaError_t e = cudaLaunchKernel(big ? aa_halo_fn<long long>(walls, odd) : aa_halo_fn<int>(walls, odd),
+                                     dim3(A.nctas + cblocks), dim3(128), hargs, 0, st);
+    if (e != cudaSuccess) return e;
+    KArgs<float> B = A;
+    B.fin = F;
+    B.fout = F;
+    B.tma = 1;
+    B.pf = 0;
+    void *args[] = {(void *)&B, (void *)&maps[0], (void *)&maps[1], (void *)&maps[2], (void *)&rc};
+    return cudaLaunchKernel(big ? aa_rows2_fn<long long>(walls, odd) : aa_rows2_fn<int>(walls, odd), dim3(A.nctas),
+                            dim3(R2_BLOCK), args, AA_STRIP_SMEM, st);
+}
 
 cudaError_t aa_plan(int precision, bool big, bool walls, bool pres, int nx, int ny, int sms, AAPlan *p)
 {

@@ -126,6 +126,13 @@ cudaError_t aa_plan(int precision, bool big, bool walls, bool pres, int nx, int 
 template <typename real>
 cudaError_t aa_step(const KArgs<real> &A, real *F, real *rho, real *side, bool walls, bool pres, bool odd, bool big,
                     const AAPlan &p, cudaStream_t st);
+// The FP32 step by row pairs in place, for channels between pressure columns:
+// A holds the strip plan (strips of at most AA_W columns, A.nctas CTAs), maps the
+// tensor maps of F with boxes of AA_SP columns by 9, 1 and 2 planes. aa_strips_plan
+// gives the resident CTAs per SM.
+cudaError_t aa_strips_plan(bool walls, bool big, int *ctas_per_sm);
+cudaError_t aa_strips_step(const KArgs<float> &A, float *F, float *rho, const CUtensorMap *maps, bool walls, bool odd,
+                           bool big, int sms, cudaStream_t st);
 cudaError_t aa_swap(int precision, void *F, bool walls, bool pres, bool big, int nx, int ny, int P, int sms,
                     cudaStream_t st);
 }  // namespace lbm

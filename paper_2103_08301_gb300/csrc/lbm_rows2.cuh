@@ -131,13 +131,6 @@ struct SmemR2 {
     int bad;
 };
 
-// Both rows of a slot at stage column sc, plane i.
-__device__ __forceinline__ float2 stage_pair(const float *slot, int i, int sc)
-{
-    return make_float2(slot[i * R2_SP + sc], slot[R2_ROW + i * R2_SP + sc]);
-}
-
-
 // One segment (strip s, fluid rows ya .. yb-1) of the row-pair step; see the
 // file comment for the schedule. The ring rows of rho / phi / lap are indexed
 // by y & (RING - 1) as in the one-row kernel.
@@ -159,6 +152,20 @@ struct MaskR2 {
     int sx;
 };
 
+// In-place streaming (AA = 1 even, 2 odd step; lbm_inplace.cu): F is source and
+// target. A node's slots are read and written by its own CTA only, so within a
+// segment the rows march as with two arrays; what other CTAs may already have
+// overwritten are the halo's populations, whose density sums come from the
+// plane `rho`, taken by a kernel before. Stage rows are 128 columns (strips of
+// at most AA_W, own columns and one neighbour each side), so every plane starts
+// on 128 bytes: the odd step brings each plane of a node's row from the row its
+// population came from, one or two planes per load (m1, m2).
+constexpr int AA_SP = 128, AA_W = 120;
+struct AAStrips {
+    const float *rho;
+    const CUtensorMap *m1, *m2;
+};
+
 // MASK: the segment of a lattice with solid nodes (lbm_mask.cu): ghost densities
 // come from MaskR2::E, solid nodes neither collide nor count, pushes along a
 // marked link bounce back. Flags are read one pair ahead, ghost densities at the
@@ -168,14 +175,25 @@ struct MaskR2 {
 // every strip on tensor loads. Without it (the batch) the wrapped columns come as
 // one 16-byte bulk copy from each end, for which nx is a multiple of 4.
 template <bool WALLS, bool PRES, bool PADDED, bool HOOK = false, typename IX = int, int EARLY = 1, bool DIRECT = false,
-          bool MASK = false>
+          bool MASK = false, int AA = 0>
 __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom<float> &G, int s, int ya, int yb,
                                                SmemR2 &S, float *stages, uint64_t *bars,
                                                RingPos2 &ring_next, const CUtensorMap *tmap, Acc<float, 1> &acc,
                                                bool &lost, bool skip_here, WrapR2 *wrap = nullptr,
-                                               const MaskR2 mk = MaskR2{})
+                                               const MaskR2 mk = MaskR2{}, const AAStrips aa = AAStrips{})
 {
     static_assert(!(DIRECT && PRES), "pressure columns have no wrapped halo");
+    static_assert(AA == 0 || (PRES && !MASK && !HOOK), "in place: channels between pressure columns");
+    constexpr int SP = AA ? AA_SP : R2_SP, ROWF = AA ? 9 * AA_SP : R2_ROW, SLOT = 2 * ROWF;
+    // both rows of a slot at stage column sc, direction i
+    auto pair_at = [&](const float *slot, int i, int sc) {
+        if constexpr (AA == 2) {  // f_i of column x lies in plane opp(i) of column x - e_i
+            const int q = opp_(i) * SP + sc - ex_(i);
+            return make_float2(slot[q], slot[ROWF + q]);
+        } else {
+            return make_float2(slot[i * SP + sc], slot[ROWF + i * SP + sc]);
+        }
+    };
     using V = float2;
     constexpr int SW = R2_BLOCK + 4;
     constexpr int PRODUCER = R2_BLOCK - 1;  // no halo duty
@@ -270,18 +288,29 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
                 // the test hook: the final pair's copy is never issued
             } else if (tid == PRODUCER && use_tma) {
                 const uint32_t st = ring_issue.s;
-                mbar_arrive_expect_tx(&bars[st], 2u * R2_TMA_ROW_BYTES);
-                float *slot = stages + (size_t)st * R2_SLOT;
+                mbar_arrive_expect_tx(&bars[st], 2u * 9u * SP * (uint32_t)sizeof(float));
+                float *slot = stages + (size_t)st * SLOT;
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
                     bool mir;
                     const int row = map_row<WALLS>(ya - 2 + 2 * q + t, ny, mir);
-                    tma_load_2d(slot + t * R2_ROW, tmap, x0 - 4, 9 * row, &bars[st]);
+                    if constexpr (AA == 2) {
+                        const int up = !WALLS && row + 1 == ny ? 0 : row + 1, dn = !WALLS && row == 0 ? ny - 1 : row - 1;
+                        float *d = slot + t * ROWF;
+                        tma_load_2d(d, aa.m2, x0 - 4, 9 * row, &bars[st]);                // planes 0, 1
+                        tma_load_2d(d + 2 * SP, aa.m1, x0 - 4, 9 * up + 2, &bars[st]);    // 2
+                        tma_load_2d(d + 3 * SP, aa.m1, x0 - 4, 9 * row + 3, &bars[st]);   // 3
+                        tma_load_2d(d + 4 * SP, aa.m1, x0 - 4, 9 * dn + 4, &bars[st]);    // 4
+                        tma_load_2d(d + 5 * SP, aa.m2, x0 - 4, 9 * up + 5, &bars[st]);    // 5, 6
+                        tma_load_2d(d + 7 * SP, aa.m2, x0 - 4, 9 * dn + 7, &bars[st]);    // 7, 8
+                    } else {
+                        tma_load_2d(slot + t * ROWF, tmap, x0 - 4, 9 * row, &bars[st]);
+                    }
                 }
             } else if (tid == PRODUCER) {
                 const uint32_t st = ring_issue.s;
                 mbar_arrive_expect_tx(&bars[st], 2u * row_bytes);
-                float *slot = stages + (size_t)st * R2_SLOT;
+                float *slot = stages + (size_t)st * SLOT;
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
                     bool mir;
@@ -317,6 +346,24 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
         }
     }
 
+    // AA: densities of pair k from the plane, where the row lies outside the segment
+    // (mirrored wall ghosts are the segment's own rows) or the column outside
+    // the strip (at and beyond a pressure column it is derived from a strip's own)
+    float hv0 = 0.f, hv1 = 0.f;
+    bool hu0 = false, hu1 = false;
+    const int hcol = dmode == 2 ? 1 : (dmode == 3 ? nx - 2 : g);
+    const bool hside = dmode == 0 && (l < 0 || l >= xw);
+    auto halo = [&](int yy, float &v, bool &use) {
+        bool mir;
+        const int row = map_row<WALLS>(yy, ny, mir);
+        use = dens && (hside || ((yy < ya || yy >= yb) && !mir));
+        if (use) v = aa.rho[(IX)row * P + hcol];
+    };
+    if constexpr (AA) {
+        halo(ya - 2, hv0, hu0);
+        halo(ya - 1, hv1, hu1);
+    }
+
     // with EARLY > 1 the first pairs go out together, so only the first wait
     // of a segment sees the full latency of a stage load (short segments)
     static_assert(EARLY >= 1 && EARLY <= R2_SLOTS, "early pairs fit the free slots");
@@ -331,7 +378,7 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
         // (1) density and phi of stencil rows yy0, yy0+1
         if (!mbar_wait_bounded(&bars[cur], ring_next.ph, poll)) lost = true;
         {
-            const float *slot = stages + (size_t)cur * R2_SLOT;
+            const float *slot = stages + (size_t)cur * SLOT;
             bool m0, m1;
             map_row<WALLS>(yy0, ny, m0);
             map_row<WALLS>(yy0 + 1, ny, m1);
@@ -340,7 +387,7 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
             if (dens) {
                 V pf[9];
 #pragma unroll
-                for (int i = 0; i < 9; ++i) pf[i] = stage_pair(slot, i, dsc);
+                for (int i = 0; i < 9; ++i) pf[i] = pair_at(slot, i, dsc);
                 if constexpr (DIRECT) {
                     if (wrapped) {
                         cp_async_wait_all();
@@ -351,6 +398,10 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
                 }
                 V sum = add_(add_(add_(pf[0], pf[1]), add_(pf[2], pf[3])), add_(add_(pf[4], pf[5]), add_(pf[6], pf[7])));
                 sum = add_(sum, pf[8]);
+                if constexpr (AA) {
+                    if (hu0) sum.x = hv0;
+                    if (hu1) sum.y = hv1;
+                }
                 if (dmode) {
                     sum.x = column_density(A, G, dmode == 3, sum.x);
                     sum.y = column_density(A, G, dmode == 3, sum.y);
@@ -359,6 +410,13 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
                 if constexpr (MASK) {
                     if (fc0 >> 15) rho_c.x = gh0;
                     if (fc1 >> 15) rho_c.y = gh1;
+                }
+                if constexpr (AA && WALLS) {
+                    // top mirror images from the ring: their rows' populations may
+                    // be overwritten while this pair is on its way
+                    if (yy0 >= ny - 1) rho_c.x = add_(S.rho[(2 * ny - 3 - yy0) & RM][tid], A.wet);
+                    if (yy0 + 1 >= ny - 1)
+                        rho_c.y = add_(yy0 == ny - 2 ? rho_c.x : S.rho[(2 * ny - 4 - yy0) & RM][tid], A.wet);
                 }
                 const V ph = eos_phi<V>(A, rho_c);
                 S.rho[r0][tid] = rho_c.x; S.rho[r1][tid] = rho_c.y;
@@ -394,10 +452,10 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
             const int b = yy0 - 2;
             const bool second = b + 1 < yb;
             const bool s0 = MASK && (fp0 >> 15), s1 = MASK && (fp1 >> 15);  // solid nodes of the pair
-            const float *slot = stages + (size_t)prev * R2_SLOT;
+            const float *slot = stages + (size_t)prev * SLOT;
             V f[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) f[i] = stage_pair(slot, i, scol);
+            for (int i = 0; i < 9; ++i) f[i] = pair_at(slot, i, scol);
             const int qm = (b - 1) & RM, q0 = b & RM, q1 = (b + 1) & RM, q2 = (b + 2) & RM;
             V ngpx, ngpy, glx, gly;
             ngrad12<V>(row3p<SW>(S.phi, qm, q0, ccol), row3p<SW>(S.phi, q0, q1, ccol), row3p<SW>(S.phi, q1, q2, ccol),
@@ -447,7 +505,24 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
             float *const out = G.fout;
             const IX oi = (IX)b * rstride + xa;  // slot of (xa, b) in plane 0
             const bool y_inner = WALLS ? (b >= 2 && b + 1 <= ny - 3) : (b >= 1 && b + 1 <= ny - 2);
-            if (x_inner && y_inner && second && !(MASK && (fp0 | fp1))) {
+            if constexpr (AA == 1) {
+                // the node's own slots, reversed; a wall link into the wall row's slot
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    if (e == 1 && !second) break;
+                    const int r = b + e;
+                    const IX ok = oi + (IX)e * rstride;
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) {
+                        const int ty = r + ey_(i), tx = xa + ex_(i);
+                        if (WALLS && (ty == 0 || ty == ny - 1)) {
+                            if (tx >= 0 && tx < nx) out[(IX)ty * rstride + i * P + tx] = el(fs[i], e);
+                        } else {
+                            out[ok + opp_(i) * P] = el(fs[i], e);
+                        }
+                    }
+                }
+            } else if (x_inner && y_inner && second && !(MASK && (fp0 | fp1))) {
                 const IX oj = oi + rstride;
                 out[oi] = fs[0].x;      out[oj] = fs[0].y;
                 out[oi + o1] = fs[1].x; out[oj + o1] = fs[1].y;
@@ -533,6 +608,12 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
                         acc.pmin = fmin(acc.pmin, pw); acc.pmax = fmax(acc.pmax, pw);
                     }
                 }
+            }
+        }
+        if constexpr (AA) {
+            if (k + 1 < npairs) {
+                halo(yy0 + 2, hv0, hu0);
+                halo(yy0 + 3, hv1, hu1);
             }
         }
         if constexpr (MASK) {
