@@ -195,7 +195,9 @@ lbm_status lbm_init(const lbm_grid *grid, const lbm_eos *eos, double tau, const 
  * (LBM_ERR_ARG), and the kernel-selection options (LBM_OPT_STAGED, ROWS2,
  * TMA, TILE, STRIP, CTAS_PER_SM, PREFETCH, PDL) affect only lbm_fields.
  * lbm_launch_info reports the step's CTAs, its threads per CTA (FP32: 128,
- * two rows each; FP64: 256), its 32 x 8 tiles as units, and no staging.
+ * two rows each; FP64: 256), its 32 x 8 tiles as units, and no staging; for
+ * long FP32 channels, which step by row pairs in place, strip rows as units
+ * and staging.
  * Errors: as lbm_init. */
 size_t lbm_workspace_bytes_inplace(const lbm_grid *grid);
 lbm_status lbm_init_inplace(const lbm_grid *grid, const lbm_eos *eos, double tau, double wetting,
@@ -277,7 +279,10 @@ typedef struct {
 lbm_status lbm_set_collision(lbm_ctx *ctx, const lbm_collision *c);
 
 /* Launch tuning and test hooks (set before stepping; changing the CTA count
- * resets the diagnostic accumulators):
+ * resets the diagnostic accumulators). FP64 grids, and FP32 grids of up to 4096
+ * nodes per SM, step by tiles of one node per thread; an explicit strip width,
+ * no staging and, in FP32, an explicit CTA count or one row per iteration select
+ * the strip kernels. All give identical results.
  *   LBM_OPT_CTAS_PER_SM  resident CTAs per SM for the step grid (0 = from
  *                        the occupancy calculator)
  *   LBM_OPT_REVERSE      nonzero: launch the step's work units in reverse CTA

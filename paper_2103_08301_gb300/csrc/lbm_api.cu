@@ -409,10 +409,19 @@ lbm_status plan_launch(lbm_ctx *ctx)
                                              (int)dyn_smem(ctx));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "smem attribute");
     }
-    // FP64: tiles (4096 x 512: 765 us by strips; see lbm_tile64.cuh). The strip
-    // kernels remain for an explicit strip width and unstaged runs.
-    if (ctx->grid.precision == 64 && ctx->allow_staged && ctx->W_opt == 0) {
-        cudaError_t e = lbm::tile64_plan(nx, ctx->grid.ny, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->sms, &ctx->t64p);
+    // Tiles (lbm_tile64.cuh): FP64 always (4096 x 512: 765 us by strips, 621 by tiles), FP32
+    // up to 4096 nodes per SM, where a row-pair CTA marches so few rows that the
+    // densities above and below its segment cost as much as its own (us per step, row
+    // pairs against tiles: 512 x 128, 7.3 and 5.3; 1024 x 256, 12.6 and 10.0; 2048 x 256,
+    // 3449 nodes per SM, 17.3 and 16.1; 2048 x 290, 3907, 18.2 and 17.7; 2048 x 320, 4312,
+    // 19.2 and 19.3; 4096 x 512, 13797, 47 and 57). The strip kernels remain for an
+    // explicit strip width or CTA count, unstaged runs and solid nodes.
+    constexpr long long TILE_NODES = 4096;
+    const bool t32 = ctx->rows2 && !ctx->big && !ctx->fault_skip && !ctx->allow_tile && ctx->ctas_per_sm_opt == 0 &&
+                     ctx->mask_host.empty() && !ctx->force_general &&
+                     (long long)nx * ctx->grid.ny <= TILE_NODES * ctx->sms;
+    if ((ctx->grid.precision == 64 || t32) && ctx->allow_staged && ctx->W_opt == 0) {
+        cudaError_t e = lbm::tile64_plan(ctx->grid.precision, nx, ctx->grid.ny, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->sms, &ctx->t64p);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy");
         ctx->t64 = true;
         ctx->nctas = ctx->t64p.ctas;
@@ -450,10 +459,9 @@ lbm_status plan_launch(lbm_ctx *ctx)
 template <typename real>
 cudaError_t launch(lbm_ctx *ctx, const lbm::KArgs<real> &A, const CUtensorMap *src_map = nullptr)
 {
-    if constexpr (sizeof(real) == 8) {
-        if (ctx->t64)
-            return lbm::tile64_launch(A, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->t64p, ctx->nctas, ctx->stream);
-    }
+    if (ctx->t64)
+        return lbm::tile64_launch<real>(A, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->t64p, ctx->nctas,
+                                        ctx->stream);
     void *fn = step_kernel_ptr(ctx);
     if (ctx->tile) {
         // one CTA per 32 x 8 tile, every stencil row staged by a tensor load
@@ -955,9 +963,9 @@ lbm_status init_ctx(const lbm_grid *grid, const lbm_eos *eos, double tau, const 
         ctx->tile_maps_ok =
             encode_population_map(&ctx->tmap_tile[0], ctx->ws + ctx->L.f0, ctx->pitch, grid->ny, lbm::T_BOX) &&
             encode_population_map(&ctx->tmap_tile[1], ctx->ws + ctx->L.f1, ctx->pitch, grid->ny, lbm::T_BOX);
+    if (wall_mask) ctx->mask_host.assign(wall_mask, wall_mask + (size_t)grid->nx * grid->ny);
     lbm_status st = plan_launch(ctx);
     if (st != LBM_OK) { lbm_free(ctx); return st; }
-    if (wall_mask) ctx->mask_host.assign(wall_mask, wall_mask + (size_t)grid->nx * grid->ny);
     st = plan_geometry(ctx);
     if (st != LBM_OK) { lbm_free(ctx); return st; }
     if (inplace) {

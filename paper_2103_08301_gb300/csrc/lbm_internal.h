@@ -150,8 +150,9 @@ namespace lbm {
 struct Tile64 {
     int th, ntx, ntiles, sx, sy, ctas, threads;
 };
-cudaError_t tile64_plan(int nx, int ny, bool walls, bool pres, bool big, int sms, Tile64 *p);
-cudaError_t tile64_launch(const KArgs<double> &A, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
+cudaError_t tile64_plan(int precision, int nx, int ny, bool walls, bool pres, bool big, int sms, Tile64 *p);
+template <typename real>
+cudaError_t tile64_launch(const KArgs<real> &A, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
                           cudaStream_t st);
 
 // Destinations of the macroscopic fields rho, ux, uy (nx ny values), tau_w, p_w

@@ -26,9 +26,10 @@ void *fields_kernel(bool walls, bool pres, bool big)
 {
     return big ? pick<real, MODE_FIELDS, long long>(walls, pres) : pick<real, MODE_FIELDS, int>(walls, pres);
 }
-void *step_kernel64(bool walls, bool pres, bool big)
+template <typename real>
+void *step_kernel_of(bool walls, bool pres, bool big)
 {
-    return big ? pick<double, MODE_STEP, long long>(walls, pres) : pick<double, MODE_STEP, int>(walls, pres);
+    return big ? pick<real, MODE_STEP, long long>(walls, pres) : pick<real, MODE_STEP, int>(walls, pres);
 }
 
 }  // namespace
@@ -38,8 +39,9 @@ void *step_kernel64(bool walls, bool pres, bool big)
 // 128 x 128 on 152 SMs that is 4, at 4096 x 512 it is 8). With walls the two rows
 // next to a wall share a tile (rows % th != 1). CTAs: a tile each up to the
 // slots of the per-CTA partials, then the resident CTAs stride over them.
-cudaError_t tile64_plan(int nx, int ny, bool walls, bool pres, bool big, int sms, Tile64 *p)
+cudaError_t tile64_plan(int precision, int nx, int ny, bool walls, bool pres, bool big, int sms, Tile64 *p)
 {
+    void *fn = precision == 64 ? step_kernel_of<double>(walls, pres, big) : step_kernel_of<float>(walls, pres, false);
     const long long rows = walls ? ny - 2 : ny;
     p->sx = pres && (nx - 1) % T64_TX == 0 ? 1 : 0;
     const long long ntx = (nx + p->sx + T64_TX - 1) / T64_TX;
@@ -60,20 +62,20 @@ cudaError_t tile64_plan(int nx, int ny, bool walls, bool pres, bool big, int sms
     const long long ntiles = ntx * ((rows + p->sy + p->th - 1) / p->th);
     p->ntiles = (int)ntiles;
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, step_kernel64(walls, pres, big),
-                                                                  T64_TX * p->th, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, T64_TX * p->th, 0);
     if (e != cudaSuccess) return e;
     p->ctas = (int)std::min<long long>(ntiles, std::min<long long>(MAX_CTAS, (long long)sms * std::max(1, occ)));
     p->threads = T64_TX * p->th;
     return cudaSuccess;
 }
 
-cudaError_t tile64_launch(const KArgs<double> &A, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
+template <typename real>
+cudaError_t tile64_launch(const KArgs<real> &A, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
                           cudaStream_t st)
 {
     T64Plan T{p.th, p.ntx, p.ntiles, p.sx, p.sy};
     void *args[] = {(void *)&A, (void *)&T};
-    return cudaLaunchKernel(step_kernel64(walls, pres, big), dim3(ctas), dim3(p.threads), args, 0, st);
+    return cudaLaunchKernel(step_kernel_of<real>(walls, pres, big), dim3(ctas), dim3(p.threads), args, 0, st);
 }
 
 namespace {
@@ -129,7 +131,7 @@ cudaError_t fields_tiles(KArgs<real> A, const FieldsOut<real> &o, bool walls, bo
     A.reverse = 0;
     A.o_rho = o.ptr[0]; A.o_vx = o.ptr[1]; A.o_vy = o.ptr[2]; A.o_tw = o.ptr[3]; A.o_pw = o.ptr[4];
     Tile64 p;
-    cudaError_t e = tile64_plan(A.nx, A.ny, walls, pres, big, sms, &p);
+    cudaError_t e = tile64_plan(sizeof(real) * 8, A.nx, A.ny, walls, pres, big, sms, &p);
     if (e != cudaSuccess) return e;
     T64Plan T{p.th, p.ntx, p.ntiles, p.sx, p.sy};
     void *args[] = {(void *)&A, (void *)&T};
@@ -150,6 +152,8 @@ cudaError_t fields_copy(const FieldsOut<real> &o, cudaStream_t st)
 }
 
 #define INST(real)                                                                                                     \
+    template cudaError_t tile64_launch<real>(const KArgs<real> &, bool, bool, bool, const Tile64 &, int,               \
+                                             cudaStream_t);                                                           \
     template void fields_route<real>(FieldsOut<real> &, int, int, const void *, size_t);                              \
     template cudaError_t fields_tiles<real>(KArgs<real>, const FieldsOut<real> &, bool, bool, bool, int, cudaStream_t); \
     template cudaError_t fields_copy<real>(const FieldsOut<real> &, cudaStream_t);

@@ -1,5 +1,5 @@
-// The FP64 step, and the fields in either precision, by tiles of 32 columns by
-// th rows, one node per thread.
+// The FP64 step, the FP32 step of small grids, and the fields in either precision,
+// by tiles of 32 columns by th rows, one node per thread.
 //
 // GB300 runs FP64 at 1/64 of the FP32 rate (two thread-instructions per clock
 // and SM), so an FP64 step is bound by each SM's FP64 pipe: what counts is the
@@ -15,6 +15,14 @@
 // kernel's within 2% (the tile's halo: densities on (32 + 4)(th + 4) points,
 // phi and Laplacian on (32 + 2)(th + 2)). The node arithmetic is the same helper
 // sequence in the same order, so the kernels give identical results.
+//
+// The FP32 step of a small grid (up to 4096 nodes per SM; both sides measured at the
+// rule, plan_launch) is bound by latency: a row-pair CTA fills its pipeline for two
+// to eight rows of its own, and pays twice the densities and potentials. A tile has
+// no pipeline to fill. 512 x 128: 7.3 us a step by row pairs, 5.3 by tiles. Launched
+// plainly: with programmatic launches, CTAs of the next step placed while this one
+// runs share SMs that the rest then do without (512 x 128: 6.2 us; 1024 x 256:
+// 11.6 against 10.0; FP64 at 128 x 128: 25 against 11).
 //
 // The FP32 fields (density, velocity, wall loads of the current state) take the
 // same kernel: they read 36 B and write 12 B per node once, with no row
@@ -58,7 +66,6 @@ __device__ __forceinline__ Row3<real> row3d(const real *a, int r, int c)
 template <typename real, bool WALLS, bool PRES, int MODE, typename IX>
 __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const KArgs<real> A, const T64Plan T)
 {
-    static_assert(sizeof(real) == 8 || MODE == MODE_FIELDS, "the FP32 step has its own kernels");
     __shared__ SmemT64<real> S;
     const int tid = threadIdx.x, tx = tid & (T64_TX - 1), ty = tid >> 5, th = T.th, tn = T64_TX * th;
     const int nx = A.nx, ny = A.ny, P = A.pitch, rstride = 9 * P;
@@ -202,7 +209,9 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
                     if (!WALLS) y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
                     out[(IX)y * rstride + i * P + x] = fs[i];
                 }
-                if constexpr (MODE == MODE_STEP) acc.mass += rho_own;
+                // FP32: the mass as a compensated FP32 pair
+                if constexpr (sizeof(real) == 4) two_sum_acc(acc.mhi, acc.mlo, rho_own);
+                else acc.mass += rho_own;
                 acc.range(rho);
             } else {
                 // outputs may be absent; wall rows and the wall loads of a
@@ -252,7 +261,7 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
                         const real tt = fma_(mul_(A.kappa, rho), -lap_of_stored<real>(S.lap[qb * T64_BW + cb]), k2p0);
                         const real pw = fma_(fma_(grx, grx, mul_(gry, gry)), mul_(real(-0.5), A.kappa), tt);
                         if (MODE == MODE_STEP) {
-                            acc.J += tw;
+                            acc.J += (double)tw;
                             acc.tmin = fmin(acc.tmin, tw); acc.tmax = fmax(acc.tmax, tw);
                             acc.pmin = fmin(acc.pmin, pw); acc.pmax = fmax(acc.pmax, pw);
                         } else {
@@ -272,9 +281,19 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
     real e[4] = {acc.tmin, acc.tmax, acc.pmin, acc.pmax};
     const bool anyw = __any_sync(0xffffffffu, e[0] < real(INFINITY) || e[1] > -real(INFINITY) ||
                                                   e[2] < real(INFINITY) || e[3] > -real(INFINITY) || acc.J != 0.0);
+    const bool wbad = __any_sync(0xffffffffu, acc.bad());
+    if constexpr (sizeof(real) == 4) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float h2 = __shfl_xor_sync(0xffffffffu, acc.mhi, o), l2 = __shfl_xor_sync(0xffffffffu, acc.mlo, o);
+            two_sum_acc(acc.mhi, acc.mlo, h2);
+            acc.mlo = __fadd_rn(acc.mlo, l2);
+        }
+        acc.mass = (double)acc.mhi + (double)acc.mlo;
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        acc.mass += __shfl_xor_sync(0xffffffffu, acc.mass, o);
+        if constexpr (sizeof(real) == 8) acc.mass += __shfl_xor_sync(0xffffffffu, acc.mass, o);
         if (anyw) {
             acc.J += __shfl_xor_sync(0xffffffffu, acc.J, o);
             e[0] = fmin(e[0], __shfl_xor_sync(0xffffffffu, e[0], o));
@@ -283,7 +302,6 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
             e[3] = fmax(e[3], __shfl_xor_sync(0xffffffffu, e[3], o));
         }
     }
-    const bool wbad = __any_sync(0xffffffffu, acc.bad());
     if (tid == 0) S.bad = 0;
     __syncthreads();
     if (lane == 0) {
