@@ -708,7 +708,10 @@ __global__ void __launch_bounds__(BLOCK) adj_local(AdjGeo<T> g, int eblocks, con
     } else {
         if (PART) {
 #pragma unroll
-            for (int i = 0; i < 9; ++i) lam[i] = gb[i] - gb[i] * g.inv_tau;
+            for (int i = 0; i < 9; ++i) {
+                if constexpr (BY_TERMS<T>) lam[i] = __fsub_rn(gb[i], __fmul_rn(gb[i], g.inv_tau));
+                else lam[i] = gb[i] - gb[i] * g.inv_tau;
+            }
         }
         m = weighted_moments(gb, g.inv_tau);
     }
@@ -718,8 +721,8 @@ __global__ void __launch_bounds__(BLOCK) adj_local(AdjGeo<T> g, int eblocks, con
     T rb, jbx, jby;
     const T usq = ux * ux + uy * uy;
     if constexpr (BY_TERMS<T>) {
-        rb = m.m0 * (T(1) - T(1.5) * usq) + T(3) * (ux * m.mx + uy * m.my) +
-             T(4.5) * (ux * ux * m.mxx + T(2) * ux * uy * m.mxy + uy * uy * m.myy);
+        rb = __fmaf_rn(T(3), ux * m.mx + uy * m.my, __fmul_rn(m.m0, T(1) - T(1.5) * usq));
+        rb = __fmaf_rn(T(4.5), ux * ux * m.mxx + T(2) * ux * uy * m.mxy + uy * uy * m.myy, rb);
         jbx = T(3) * m.mx + T(9) * (ux * m.mxx + uy * m.mxy) - T(3) * ux * m.m0;
         jby = T(3) * m.my + T(9) * (ux * m.mxy + uy * m.myy) - T(3) * uy * m.m0;
         rb -= jbx * ux + jby * uy;
@@ -1068,12 +1071,16 @@ __global__ void __launch_bounds__(TX * TMAX) adj_finish_terms(AdjGeo<float> g, i
         const int c = px - x0 + 1, r = py - y0 + 1;
         return c >= 0 && c < BW && r >= 0 && r < th + 2 ? S[r * BW + c] : T(0);
     };
+    // the point's own part; here and below, which products are fused is fixed,
+    // since the compiler's choice differs between branches
+    auto own = [](T pb, T dp, T lb) {
+        return __fmaf_rn(-(T(6) * (T(1) - wq<T>(0))), lb, __fmul_rn(pb, dp));
+    };
     // Ebar at the extended point (px, py), whose density has dphi = dp
     auto ebar = [&](int px, int py, T dp) {
         T eb = 0;
         if (px >= -1 && px <= nx && py >= -1 && py <= ny) {
-            eb += at(SP, px, py) * dp;
-            eb -= T(6) * (T(1) - wq<T>(0)) * at(SL, px, py);
+            eb = own(at(SP, px, py), dp, at(SL, px, py));
         }
 #pragma unroll
         for (int i = 1; i < 9; ++i) {
@@ -1083,9 +1090,9 @@ __global__ void __launch_bounds__(TX * TMAX) adj_finish_terms(AdjGeo<float> g, i
                 T s = 0;
                 if (ex_(i) != 0) s += T(ex_(i)) * C[0];
                 if (ey_(i) != 0) s += T(ey_(i)) * C[nx];
-                eb += T(3) * wq<T>(i) * s;
+                eb = __fmaf_rn(T(3) * wq<T>(i), s, eb);
             }
-            if (qx >= -1 && qx <= nx && qy >= -1 && qy <= ny) eb += T(6) * wq<T>(i) * at(SL, qx, qy);
+            if (qx >= -1 && qx <= nx && qy >= -1 && qy <= ny) eb = __fmaf_rn(T(6) * wq<T>(i), at(SL, qx, qy), eb);
         }
         return eb;
     };
@@ -1107,10 +1114,9 @@ __global__ void __launch_bounds__(TX * TMAX) adj_finish_terms(AdjGeo<float> g, i
     } else {
         // away from the walls: no objective source, every neighbour on the ring
         const T *l = SL + (ty + 1) * BW + tx + 1;
-        s += SP[(ty + 1) * BW + tx + 1] * dphi[cn];
-        s -= T(6) * (T(1) - wq<T>(0)) * l[0];
+        s = own(SP[(ty + 1) * BW + tx + 1], dphi[cn], l[0]);
 #pragma unroll
-        for (int i = 1; i < 9; ++i) s += T(6) * wq<T>(i) * l[-ey_(i) * BW - ex_(i)];
+        for (int i = 1; i < 9; ++i) s = __fmaf_rn(T(6) * wq<T>(i), l[-ey_(i) * BW - ex_(i)], s);
     }
     T rb = rl + s;
     if (x == 1 || x == nx - 2) {
