@@ -719,15 +719,20 @@ __global__ void __launch_bounds__(BLOCK) adj_local(AdjGeo<T> g, int eblocks, con
     // e_i: with s = M u (second moments), u_eq-bar / rho = 3 m + 9 s - 3 u m0
     // and rho-bar - u_eq-bar . u_eq / rho = m0 (1 + 1.5 u^2) - 4.5 u.s
     T rb, jbx, jby;
-    const T usq = ux * ux + uy * uy;
     if constexpr (BY_TERMS<T>) {
-        rb = __fmaf_rn(T(3), ux * m.mx + uy * m.my, __fmul_rn(m.m0, T(1) - T(1.5) * usq));
-        rb = __fmaf_rn(T(4.5), ux * ux * m.mxx + T(2) * ux * uy * m.mxy + uy * uy * m.myy, rb);
-        jbx = T(3) * m.mx + T(9) * (ux * m.mxx + uy * m.mxy) - T(3) * ux * m.m0;
-        jby = T(3) * m.my + T(9) * (ux * m.mxy + uy * m.myy) - T(3) * uy * m.m0;
-        rb -= jbx * ux + jby * uy;
+        // every product that is fused is named: the compiler's choice depends on
+        // the code around it
+        auto dot = [](T a, T b, T c, T d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); };
+        const T ux2 = __fmul_rn(ux, ux), uy2 = __fmul_rn(uy, uy), uxy = __fmul_rn(T(2) * ux, uy);
+        const T usq = __fadd_rn(ux2, uy2);
+        rb = dot(T(3), dot(ux, m.mx, uy, m.my), m.m0, __fmaf_rn(T(-1.5), usq, T(1)));
+        rb = __fmaf_rn(T(4.5), __fmaf_rn(uy2, m.myy, dot(ux2, m.mxx, uxy, m.mxy)), rb);
+        jbx = __fmaf_rn(-__fmul_rn(T(3), ux), m.m0, dot(T(3), m.mx, T(9), dot(ux, m.mxx, uy, m.mxy)));
+        jby = __fmaf_rn(-__fmul_rn(T(3), uy), m.m0, dot(T(3), m.my, T(9), dot(ux, m.mxy, uy, m.myy)));
+        rb = __fsub_rn(rb, dot(jbx, ux, jby, uy));
     } else {
         const T sx = ux * m.mxx + uy * m.mxy, sy = ux * m.mxy + uy * m.myy;
+        const T usq = ux * ux + uy * uy;
         rb = m.m0 * (T(1) + T(1.5) * usq) - T(4.5) * (ux * sx + uy * sy);
         jbx = T(3) * (m.mx - ux * m.m0) + T(9) * sx;
         jby = T(3) * (m.my - uy * m.m0) + T(9) * sy;
