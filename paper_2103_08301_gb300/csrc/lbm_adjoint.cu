@@ -1427,7 +1427,7 @@ lbm_status adj_run_chain(lbm_adjoint *a, const Run &r, int buf, cudaStream_t st,
 // states. Preparing run i + 1 (recomputing its block's states first, where it
 // opens one: by then the fields of every state in their storage are taken)
 // does not depend on the adjoint, so it overlaps the chain of run i, whose two
-// short kernels per step leave half of the FP64 pipe idle (512 x 128, 200 steps
+// short kernels per step leave most of the FP64 pipe idle (512 x 128, 200 steps
 // forward and back: 14.1 ms one after the other, 11.4 overlapped; 1024 x 256
 // with an FP32 reverse, 100 steps: 6.2 and 5.7). Run i's fields lie in buffer
 // i & 1, free again once chain i - 2 is through.

@@ -29,7 +29,7 @@
 // pass, 36 B read, 36 B written and 4 B of densities read by the step, 116 B
 // against the two-array step's 72 B; storage 40 B against 72 B. Large FP32
 // channels between pressure columns step by row pairs instead, with densities
-// from the plane for the halo only (aa_step_kernel_rows2): about 76 B.
+// from the plane for the halo only (aa_step_kernel_rows2): about 74 B.
 
 #include <cuda_runtime.h>
 
@@ -728,8 +728,8 @@ __global__ void __launch_bounds__(AA2_THREADS, LBM_AA2_MIN_BLOCKS)
 // segment reads outside itself come from the plane: four columns around every
 // strip boundary and four rows around every cut, about a twentieth of the
 // lattice, instead of a density pass over all of it. 16384 x 2048: 0.837 ms a step
-// by tiles (density pass 0.211 of it), 0.668 by row pairs; the two-array step, with
-// 40 bytes a node less to move than the tiles and 4 less than this, 0.472.
+// by tiles (density pass 0.211 of it), 0.668 by row pairs; the two-array step, which
+// moves 72 B a node against 116 and 74, 0.472.
 // ---------------------------------------------------------------------------
 
 template <bool ODD, typename IX>

@@ -8,8 +8,9 @@ kappa = 0.5, seeded synthetic initial density.
   python -m paper_2103_08301_gb300.profile_step --nx 4096 --ny 2048 --steps 5 [--precision 32] [--mask]
       [--inplace]
 
-Prints the mean step time and effective bandwidth (72 B/node in FP32; 116
-B/node for an in-place context, whose step is a density pass and a collide pass).
+Prints the mean step time and effective bandwidth (72 B/node in FP32; for an
+in-place context 116 B/node by tiles, a density pass and a collide pass, or about
+74 by row pairs).
 """
 from __future__ import annotations
 
@@ -66,7 +67,8 @@ def main():
         ms = a.elapsed_time(b) / args.steps
         info = lat.launch_info()
         nan = lat.diag()["nan_detected"]
-    bpn = (116 if args.inplace else 72) if args.precision == 32 else (232 if args.inplace else 144)
+    fp32 = (74 if info["staged"] else 116) if args.inplace else 72
+    bpn = fp32 if args.precision == 32 else (232 if args.inplace else 144)
     print(json.dumps({"nx": nx, "ny": ny, "precision": args.precision, "inplace": args.inplace, "ms_per_step": ms,
                       "GBps": bpn * nx * ny / ms / 1e6, "MLUPS": nx * ny / ms / 1e3,
                       "launch": info, "nan": nan}))
