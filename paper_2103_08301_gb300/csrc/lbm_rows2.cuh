@@ -347,12 +347,14 @@ __device__ __forceinline__ void run_segment_r2(const KArgs<float> &A, const Geom
     }
 
     // AA: densities of pair k from the plane, where the row lies outside the segment
-    // (mirrored wall ghosts are the segment's own rows) or the column outside
-    // the strip (at and beyond a pressure column it is derived from a strip's own)
+    // (mirrored wall ghosts are the segment's own rows) or the column that a density
+    // comes from outside the strip. That is the lane's own column, or at and beyond a
+    // pressure column its interior neighbour: nx-2 belongs to the next strip where
+    // the last one is two columns wide.
     float hv0 = 0.f, hv1 = 0.f;
     bool hu0 = false, hu1 = false;
     const int hcol = dmode == 2 ? 1 : (dmode == 3 ? nx - 2 : g);
-    const bool hside = dmode == 0 && (l < 0 || l >= xw);
+    const bool hside = hcol < x0 || hcol >= x0 + xw;
     auto halo = [&](int yy, float &v, bool &use) {
         bool mir;
         const int row = map_row<WALLS>(yy, ny, mir);
