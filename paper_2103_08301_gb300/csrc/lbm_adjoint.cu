@@ -628,7 +628,11 @@ __device__ __forceinline__ Mom<T> weighted_moments(const T (&v)[9], T scale)
 }
 
 // Programmatic dependent launch (lbm_rows2.cuh): wait for the kernel before,
-// then let the next one's launch overlap this one.
+// then let the next one's launch overlap this one. A grid may thus be resident
+// while the one before still writes its inputs. Those inputs are plain pointers:
+// const __restrict__ would promise that they do not change while the grid lives,
+// and allow loads from the read-only cache, or ahead of the wait. The state's
+// fields (fld) are complete before a run's first grid starts (adj_chain_t).
 __device__ __forceinline__ void chain_start()
 {
     lbm::griddep_wait();
@@ -650,7 +654,7 @@ __device__ __forceinline__ void chain_start()
 // would slow two of every sixteen warps of a 512-wide row, always on the same
 // SMs (51k cycles on the busiest SM against 29k on average).
 template <typename T, bool PART, int BLOCK>
-__global__ void __launch_bounds__(BLOCK) adj_local(AdjGeo<T> g, int eblocks, const T *__restrict__ lam_in,
+__global__ void __launch_bounds__(BLOCK) adj_local(AdjGeo<T> g, int eblocks, const T *lam_in,
                                                    const T *__restrict__ fld, T *lam_out, T *Ax, T *Ay,
                                                    T *Jbx, T *Jby, T *R, T *Cw, double *AS)
 {
@@ -843,10 +847,8 @@ __global__ void __launch_bounds__(BLOCK) adj_local(AdjGeo<T> g, int eblocks, con
 // the rest is one wave's load, two barriers and the launch).
 template <typename T, bool PART>
 __global__ void __launch_bounds__(TX * TMAX) adj_finish(AdjGeo<T> g, int th, const T *__restrict__ fld,
-                                                        const T *__restrict__ Ax, const T *__restrict__ Ay,
-                                                        const T *__restrict__ Jbx, const T *__restrict__ Jby,
-                                                        const T *__restrict__ R, const T *__restrict__ Cw, T *lam_out,
-                                                        double *colp)
+                                                        const T *Ax, const T *Ay, const T *Jbx, const T *Jby,
+                                                        const T *R, const T *Cw, T *lam_out, double *colp)
 {
     __shared__ T SX[SMEM_A], SY[SMEM_A], BX[SMEM_A], BY[SMEM_A], SL[SMEM_B];
     chain_start();
@@ -996,13 +998,9 @@ __global__ void __launch_bounds__(TX * TMAX) adj_finish(AdjGeo<T> g, int th, con
 // beyond the ghost row or the column Lbar is zero.
 template <bool PART>
 __global__ void __launch_bounds__(TX * TMAX) adj_finish_terms(AdjGeo<float> g, int th, const float *__restrict__ fld,
-                                                              const float *__restrict__ Ax,
-                                                              const float *__restrict__ Ay,
-                                                              const float *__restrict__ Jbx,
-                                                              const float *__restrict__ Jby,
-                                                              const float *__restrict__ R,
-                                                              const float *__restrict__ Cw, float *lam_out,
-                                                              double *colp)
+                                                              const float *Ax, const float *Ay, const float *Jbx,
+                                                              const float *Jby, const float *R, const float *Cw,
+                                                              float *lam_out, double *colp)
 {
     using T = float;
     __shared__ T SX[SMEM_A], SY[SMEM_A], SR[SMEM_A], SL[SMEM_B], SP[SMEM_B];
@@ -1298,10 +1296,10 @@ States block_states(lbm_adjoint *a, int64_t b)
 template <typename T>
 T *as(double *p) { return reinterpret_cast<T *>(p); }
 
-// Launch with programmatic stream serialization: the kernel's launch overlaps
-// the previous kernel of the chain, which it waits for before any access.
+// Launch with programmatic stream serialization (`chained`): the kernel's launch
+// overlaps the previous kernel of the chain, which it waits for before any access.
 template <typename... P, typename... Q>
-cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, Q &&...q)
+cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t st, bool chained, Q &&...q)
 {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1311,7 +1309,7 @@ cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t 
     cfg.blockDim = block;
     cfg.stream = st;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chained ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, k, static_cast<P>(q)...);
 }
 
@@ -1393,14 +1391,16 @@ lbm_status adj_chain_t(lbm_adjoint *a, const Run &r, int buf, cudaStream_t st, d
     for (int m = r.m1 - 1; m >= r.m0; --m) {
         const T *f = as<T>(a->fld[buf]) + (size_t)(m - r.m0) * NFIELD * N;
         T *li = as<T>(lin), *lo = as<T>(lout);
-        ACK(launch_chained(adj_local<T, PART, LB>, dim3(nblocks), dim3(LB), st, g, (int)eblocks, li, f, lo,
+        // a run's first kernel is launched plainly: its fields were written by
+        // the kernels or events before it in the stream
+        ACK(launch_chained(adj_local<T, PART, LB>, dim3(nblocks), dim3(LB), st, m + 1 < r.m1, g, (int)eblocks, li, f, lo,
                            as<T>(a->Ax), as<T>(a->Ay), as<T>(a->Jbx), as<T>(a->Jby), as<T>(a->R), as<T>(a->Cw), a->AS),
             "adjoint local kernel");
         auto finish = adj_finish<T, PART>;
         if constexpr (BY_TERMS<T>) {
             if (g.walls && g.bc_x) finish = adj_finish_terms<PART>;
         }
-        ACK(launch_chained(finish, dim3(tg), dim3(TX * th), st, g, th, f, as<T>(a->Ax), as<T>(a->Ay), as<T>(a->Jbx),
+        ACK(launch_chained(finish, dim3(tg), dim3(TX * th), st, true, g, th, f, as<T>(a->Ax), as<T>(a->Ay), as<T>(a->Jbx),
                            as<T>(a->Jby), as<T>(a->R), as<T>(a->Cw), lo, a->colp),
             "adjoint finish kernel");
         std::swap(lin, lout);
