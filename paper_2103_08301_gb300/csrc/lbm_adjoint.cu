@@ -993,9 +993,9 @@ __global__ void __launch_bounds__(TX * TMAX) adj_finish(AdjGeo<T> g, int th, con
 // three kernels of 26 us together became this one), the terms of
 // every sum added one by one: Lbar and phibar on the ring around the tile,
 // Ebar at this node's points of the ghost-extended lattice (itself, its mirror
-// images behind the walls), then their sum. The host keeps the two rows next
-// to a wall in one tile (rows % th != 1), whose ring then holds all of it:
-// beyond the ghost row or the column Lbar is zero.
+// images behind the walls), then their sum. Only for tile heights that keep the
+// two rows next to a wall in one tile (rows % th != 1), whose ring then holds all
+// of it: beyond the ghost row or the column Lbar is zero.
 template <bool PART>
 __global__ void __launch_bounds__(TX * TMAX) adj_finish_terms(AdjGeo<float> g, int th, const float *__restrict__ fld,
                                                               const float *Ax, const float *Ay, const float *Jbx,
@@ -1348,7 +1348,7 @@ int tile_rows(const lbm_adjoint *a, int states)
     int best = 8;
     long long least = -1;
     for (int th = 4; th <= TMAX; ++th) {
-        if (rows % th == 1) continue;  // adj_finish_terms: the two rows next to a wall share a tile
+        if (rows % th == 1) continue;  // adj_finish_terms: the two rows next to a wall share a tile (adj_chain_t)
         const long long t = ntx * ((rows + th - 1) / th) * states, cost = (t + a->sms - 1) / a->sms * (th + 2);
         if (least < 0 || cost < least) { least = cost; best = th; }
     }
@@ -1398,7 +1398,8 @@ lbm_status adj_chain_t(lbm_adjoint *a, const Run &r, int buf, cudaStream_t st, d
             "adjoint local kernel");
         auto finish = adj_finish<T, PART>;
         if constexpr (BY_TERMS<T>) {
-            if (g.walls && g.bc_x) finish = adj_finish_terms<PART>;
+            // where every height leaves a single row (rows = 1 mod 720720): adj_finish
+            if (g.walls && g.bc_x && (g.ny - 2) % th != 1) finish = adj_finish_terms<PART>;
         }
         ACK(launch_chained(finish, dim3(tg), dim3(TX * th), st, true, g, th, f, as<T>(a->Ax), as<T>(a->Ay), as<T>(a->Jbx),
                            as<T>(a->Jby), as<T>(a->R), as<T>(a->Cw), lo, a->colp),
