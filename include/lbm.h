@@ -221,9 +221,10 @@ lbm_status lbm_step(lbm_ctx *ctx, int64_t n);
  *                for pressure columns and channels without walls.
  * Each pointer may be NULL (skipped), a device pointer or a host pointer, of
  * the context precision. Destinations in the current device's memory, aligned
- * to their elements, are written by the kernel; the others go through a device
- * scratch of their size, allocated at the first call that needs it and kept
- * (with a wall mask also for skipped outputs). Synchronises the stream. */
+ * to their elements and within one allocation, are written by the kernel; the
+ * others go through a device scratch of their size, allocated at the first call
+ * that needs it and kept (with a wall mask also for skipped outputs).
+ * Synchronises the stream. */
 lbm_status lbm_fields(lbm_ctx *ctx, void *rho, void *ux, void *uy, void *tau_wall,
                       void *p_wall);
 

@@ -157,8 +157,8 @@ cudaError_t tile64_launch(const KArgs<real> &A, bool walls, bool pres, bool big,
 
 // Destinations of the macroscopic fields rho, ux, uy (nx ny values), tau_w, p_w
 // (2 nx), any of them NULL. fields_route decides which a kernel writes itself
-// (device memory of this device that overlaps neither another output nor the
-// `busy` range, the state): ptr = dst; the others need `scratch` bytes, output
+// (memory of this device, in one allocation, that overlaps neither another output
+// nor the `busy` range, the state): ptr = dst; the others need `scratch` bytes, output
 // k at offset[k], which the caller points ptr[k] to. fields_tiles computes the
 // outputs with a ptr; fields_copy brings the scratch ones to their destinations.
 template <typename real>

@@ -1,4 +1,7 @@
-// The FP64 step and the fields by tiles (lbm_tile64.cuh): plan and launch.
+// The step of FP64 and of small FP32 grids, and the fields, by tiles
+// (lbm_tile64.cuh): plan and launch.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -80,18 +83,40 @@ cudaError_t tile64_launch(const KArgs<real> &A, bool walls, bool pres, bool big,
 
 namespace {
 
-// Whether a kernel may write `bytes` at p itself: memory of the current device,
-// aligned to its elements.
-bool writable_here(const void *p, size_t align)
+// cuPointerGetAttributes from the driver, looked up once through the runtime.
+PFN_cuPointerGetAttributes_v7000 pointer_attributes()
 {
-    cudaPointerAttributes at{};
-    int dev = 0;
-    if ((uintptr_t)p % align != 0 || cudaGetDevice(&dev) != cudaSuccess) return false;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice && at.device == dev;
+    static const PFN_cuPointerGetAttributes_v7000 fn = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &p, 7000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        return reinterpret_cast<PFN_cuPointerGetAttributes_v7000>(p);
+    }();
+    return fn;
+}
+
+// Whether a kernel may write `bytes` at p itself: memory of device `dev`, aligned
+// to its elements, all of it in one allocation. A range that leaves its allocation
+// goes the way of host destinations, whose copy refuses it.
+bool writable_here(const void *p, size_t bytes, size_t align, int dev)
+{
+    const PFN_cuPointerGetAttributes_v7000 query = pointer_attributes();
+    if ((uintptr_t)p % align != 0 || !query) return false;
+    unsigned type = 0, managed = 0;
+    int ordinal = -1;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute at[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                 CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *data[5] = {&type, &managed, &ordinal, &start, &size};
+    if (query(5, at, data, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    return type == CU_MEMORYTYPE_DEVICE && !managed && ordinal == dev && (CUdeviceptr)p >= start &&
+           (CUdeviceptr)p - start <= size && bytes <= size - (size_t)((CUdeviceptr)p - start);
 }
 bool overlap(const void *a, size_t na, const void *b, size_t nb)
 {
@@ -104,11 +129,13 @@ template <typename real>
 void fields_route(FieldsOut<real> &o, int nx, int ny, const void *busy, size_t busy_bytes)
 {
     const size_t N = (size_t)nx * ny * sizeof(real), W = 2 * (size_t)nx * sizeof(real);
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
     o.scratch = 0;
     for (int k = 0; k < 5; ++k) {
         const size_t bytes = k < 3 ? N : W;
         o.bytes[k] = bytes;
-        bool direct = o.dst[k] && writable_here(o.dst[k], sizeof(real)) && !overlap(o.dst[k], bytes, busy, busy_bytes);
+        bool direct = o.dst[k] && writable_here(o.dst[k], bytes, sizeof(real), dev) && !overlap(o.dst[k], bytes, busy, busy_bytes);
         for (int j = 0; direct && j < 5; ++j)
             if (j != k && o.dst[j] && overlap(o.dst[k], bytes, o.dst[j], j < 3 ? N : W)) direct = false;
         o.ptr[k] = direct ? (real *)o.dst[k] : nullptr;
