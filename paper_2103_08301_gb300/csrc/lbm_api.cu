@@ -360,6 +360,16 @@ int band_rows(int nyf, int nstrips, int nctas, int walls)
     return std::max(1, band);
 }
 
+// CTAs of the strip plan with per_sm of them resident on an SM, and its bands.
+void plan_strip_ctas(lbm_ctx *ctx, int per_sm)
+{
+    long long n = (long long)ctx->sms * per_sm;
+    n = std::min<long long>(n, std::max<long long>(1, ctx->units / 2));
+    n = std::min<long long>(n, lbm::MAX_CTAS);
+    ctx->nctas = (int)std::max<long long>(1, n);
+    ctx->band = band_rows(ctx->nyf, ctx->nstrips, ctx->nctas, ctx->grid.walls);
+}
+
 // Strip partition and the CTA count of the step grid.
 lbm_status plan_launch(lbm_ctx *ctx)
 {
@@ -398,11 +408,7 @@ lbm_status plan_launch(lbm_ctx *ctx)
         if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy");
         per_sm = std::max(1, occ);
     }
-    long long n = (long long)ctx->sms * per_sm;
-    n = std::min<long long>(n, std::max<long long>(1, ctx->units / 2));
-    n = std::min<long long>(n, lbm::MAX_CTAS);
-    ctx->nctas = (int)std::max<long long>(1, n);
-    ctx->band = band_rows(ctx->nyf, ctx->nstrips, ctx->nctas, ctx->grid.walls);
+    plan_strip_ctas(ctx, per_sm);
     if (ctx->rows2 && !ctx->big && ctx->units < EARLY_ROWS * ctx->nctas) {
         ctx->early = true;
         cudaError_t e = cudaFuncSetAttribute(step_kernel_ptr(ctx), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -835,10 +841,17 @@ lbm_status plan_geometry(lbm_ctx *ctx)
     ctx->mask_rows2 = false;
     if (st != LBM_OK || !ctx->mask) return st;
     if (ctx->rows2 && !ctx->big) {
-        // the row-pair plan holds where as many CTAs stay resident
-        int per_sm = 0;
-        cudaError_t e = lbm::mask_rows2_plan(ctx->mask, ctx->early, &per_sm);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "mask step plan");
+        // the strip plan with this kernel's own residency
+        ctx->tile = false;
+        int per_sm = ctx->ctas_per_sm_opt;
+        for (bool early : {false, true}) {
+            int occ = 0;
+            cudaError_t e = lbm::mask_rows2_plan(ctx->mask, early, &occ);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "mask step plan");
+            if (ctx->ctas_per_sm_opt <= 0) per_sm = early ? std::min(per_sm, std::max(1, occ)) : std::max(1, occ);
+        }
+        plan_strip_ctas(ctx, per_sm);
+        ctx->early = ctx->units < EARLY_ROWS * ctx->nctas;
         ctx->mask_rows2 = true;
         return LBM_OK;
     }
