@@ -359,9 +359,12 @@ typedef enum {
 } lbm_option;
 lbm_status lbm_set_option(lbm_ctx *ctx, lbm_option opt, int64_t value);
 /* Launch geometry of the step kernel: CTAs, threads per CTA, work units and
- * whether the staged variant runs (FP64 tiles, which need no stage, count as
- * staged; with a wall mask: the threads of the general-geometry kernels, not
- * staged). Any output may be NULL. */
+ * whether the staged variant runs. Units are strip rows, or tiles where the step
+ * runs by tiles (FP64 and small FP32 grids; they need no stage and count as
+ * staged). With solid nodes: the geometry of the general-geometry kernels (a node
+ * per thread, nodes as units, not staged), which the fields, FP64 steps and FP32
+ * steps without row pairs run; an FP32 step by row pairs is not reported. Any
+ * output may be NULL. */
 lbm_status lbm_launch_info(const lbm_ctx *ctx, int64_t *ctas, int64_t *threads, int64_t *units,
                            int64_t *staged);
 

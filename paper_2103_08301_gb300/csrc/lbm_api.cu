@@ -1380,10 +1380,18 @@ lbm_status lbm_launch_info(const lbm_ctx *ctx, int64_t *ctas, int64_t *threads, 
         if (staged) *staged = 0;
         return LBM_OK;
     }
+    if (ctx->mask) {
+        // the general-geometry kernels, a node per thread, also where FP32 steps by row pairs
+        if (ctas) *ctas = lbm::mask_blocks(ctx->mask);
+        if (threads) *threads = 256;
+        if (units) *units = (int64_t)ctx->grid.nx * ctx->grid.ny;
+        if (staged) *staged = 0;
+        return LBM_OK;
+    }
     if (ctas) *ctas = ctx->nctas;
-    if (threads) *threads = ctx->mask ? 256 : threads_of(ctx);
-    if (units) *units = ctx->mask ? (int64_t)ctx->grid.nx * ctx->grid.ny : ctx->units;
-    if (staged) *staged = (ctx->staged && !ctx->mask) ? 1 : 0;
+    if (threads) *threads = threads_of(ctx);
+    if (units) *units = ctx->t64 ? ctx->t64p.ntiles : (ctx->tile ? ctx->nctas : ctx->units);
+    if (staged) *staged = ctx->staged ? 1 : 0;
     return LBM_OK;
 }
 
