@@ -50,7 +50,12 @@ struct SmemT64 {
 
 // Tile grid: th rows per tile, shifted one column left when the outlet column
 // would open a tile (its stencil is its neighbour's), one row down when no height
-// keeps the two rows next to a wall in one tile.
+// keeps the two rows next to a wall in one tile. CTAs stride over the tiles row of
+// tiles by row of tiles. A tile with a pressure column costs more (its lanes
+// extrapolate besides), and a stride that is a multiple of ntx (456 CTAs over 3, 4,
+// 6, 8, 12 columns of tiles) would give such tiles to the same CTAs always: each row
+// of tiles starts one tile further on (FP64, 97 x 60000: 3283 us a step without, 2611
+// with; 250 x 24000: 2619 and 1827; 4096 x 512: 563 and 551).
 struct T64Plan {
     int th, ntx, ntiles, sx, sy;
 };
@@ -91,7 +96,12 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
 
     for (int t = cta; t < T.ntiles; t += gridDim.x) {
         const int by = t / T.ntx;
-        const int x0 = (t - by * T.ntx) * T64_TX - T.sx, y0 = yf0 + by * th - T.sy;
+        int bx = t - by * T.ntx;
+        if (PRES && T.ntiles > (int)gridDim.x) {  // see T64Plan
+            bx += by % T.ntx;
+            if (bx >= T.ntx) bx -= T.ntx;
+        }
+        const int x0 = bx * T64_TX - T.sx, y0 = yf0 + by * th - T.sy;
         const int xa = x0 + tx, r = y0 + ty;
         const bool active = xa >= 0 && xa < nx && r >= yf0 && r < yf1;
         const bool pin = PRES && active && xa == 0, pout = PRES && active && xa == nx - 1;
