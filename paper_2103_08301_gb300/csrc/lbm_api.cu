@@ -382,15 +382,29 @@ lbm_status plan_launch(lbm_ctx *ctx)
     // multiple of 4)
     ctx->rows2 = ctx->allow_rows2 && ctx->staged && ctx->grid.precision == 32 &&
                  lbm::cols_per_thread<float, true>() == 1;
-    if (ctx->rows2) {
-        const int W2 = lbm::strip_width(nx, std::min(wmax, lbm::R2_W), ctx->grid.bc_x);
-        if (W2 % 4 == 0) W = W2;
-        else ctx->rows2 = false;
-    }
-    ctx->W = W;
-    ctx->nstrips = (nx + W - 1) / W;
+    const int W2 = ctx->rows2 ? lbm::strip_width(nx, std::min(wmax, lbm::R2_W), ctx->grid.bc_x) : 0;
+    if (W2 % 4 != 0) ctx->rows2 = false;
+    const bool plain = ctx->mask_host.empty() && !ctx->force_general;  // no solid nodes
+    constexpr long long TILE_NODES = 4096;  // see below
+    const bool t32 = ctx->rows2 && !ctx->big && !ctx->fault_skip && !ctx->allow_tile && ctx->ctas_per_sm_opt == 0 &&
+                     plain && ctx->W_opt == 0 && (long long)nx * ctx->grid.ny <= TILE_NODES * ctx->sms;
     ctx->yf0 = ctx->grid.walls ? 1 : 0;
     ctx->nyf = ctx->grid.walls ? ctx->grid.ny - 2 : ctx->grid.ny;
+    if (ctx->rows2 && plain && !t32 && !ctx->allow_tile && !ctx->grid.bc_x && nx % 4 != 0) {
+        // Odd periodic widths that one or two strips of one row a thread (128 columns)
+        // hold, but not as many of row pairs (124). Us per step, row pairs against one
+        // row: 125 x 48000, 167 and 125 (walls: 184 and 132); 125 x 6400, 30 and 29 (33
+        // and 30). With two strips against three it depends on the rows that a CTA
+        // marches: 250 x 3200, 13 rows, 26 and 28 (27 and 33); 250 x 8000, 32 rows, 49
+        // and 51 (55 and 52); 250 x 24000, 95 rows, 126 and 122 (144 and 128). From
+        // three on row pairs are as fast or faster (381 x 15748: 111 and 123; 128 and 128).
+        const int n1 = (nx + W - 1) / W, n2 = (nx + W2 - 1) / W2;
+        const long long rows = (long long)n2 * ctx->nyf / (5 * ctx->sms);
+        if (n2 > n1 && (n1 == 1 || (n1 == 2 && rows >= (ctx->grid.walls ? 24 : 64)))) ctx->rows2 = false;
+    }
+    if (ctx->rows2) W = W2;
+    ctx->W = W;
+    ctx->nstrips = (nx + W - 1) / W;
     ctx->units = (long long)ctx->nstrips * ctx->nyf;
     ctx->early = false;  // chosen once the CTA count is known
     ctx->t64 = false;    // likewise
@@ -422,10 +436,6 @@ lbm_status plan_launch(lbm_ctx *ctx)
     // 3449 nodes per SM, 17.3 and 16.1; 2048 x 290, 3907, 18.2 and 17.7; 2048 x 320, 4312,
     // 19.2 and 19.3; 4096 x 512, 13797, 47 and 57). The strip kernels remain for an
     // explicit strip width or CTA count, unstaged runs and solid nodes.
-    constexpr long long TILE_NODES = 4096;
-    const bool t32 = ctx->rows2 && !ctx->big && !ctx->fault_skip && !ctx->allow_tile && ctx->ctas_per_sm_opt == 0 &&
-                     ctx->mask_host.empty() && !ctx->force_general &&
-                     (long long)nx * ctx->grid.ny <= TILE_NODES * ctx->sms;
     if ((ctx->grid.precision == 64 || t32) && ctx->allow_staged && ctx->W_opt == 0) {
         cudaError_t e = lbm::tile64_plan(ctx->grid.precision, nx, ctx->grid.ny, ctx->grid.walls, ctx->grid.bc_x, ctx->big, ctx->sms, &ctx->t64p);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "occupancy");
