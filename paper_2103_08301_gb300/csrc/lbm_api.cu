@@ -351,12 +351,27 @@ int threads_of(const lbm_ctx *ctx)
 // whole column, i.e. strip-major order, when there are fewer CTAs than
 // strips). With walls no band boundary may fall between fluid rows 1|2 or
 // ny-3|ny-2 (fluid offsets 1 and nyf-1).
+//
+// A segment costs its rows and about five more for its halo, so the last band must
+// not be a few rows only: its CTAs would march through many short segments, and the
+// step waits for them. Higher bands than the share cost too (a CTA's rows then lie
+// in two strips, out of step with their neighbours: 14491 x 1739, share 268, a band
+// of 290 takes 443 us a step instead of 355), hence the weights below. FP32 row
+// pairs, us per step with the share itself and with the band chosen: 1999 x 1500,
+// last band of 4 rows, 58.6 and 51.1 (walls: 2 rows, 79.9 and 57.6); 5343 x 1244,
+// 3 rows, 143 and 98.6; 1180 x 741, 1 row, 37.4 and 21.2. 16384 x 2048 keeps its 359.
 int band_rows(int nyf, int nstrips, int nctas, int walls)
 {
     const long long share = ((long long)nyf * nstrips + nctas - 1) / nctas;
-    int band = (int)std::min<long long>(nyf, std::max<long long>(8, share));
-    if (walls)
-        while (band < nyf && (nyf - 1) % band == 0) ++band;
+    const int least = (int)std::min<long long>(nyf, std::max<long long>(8, share));
+    int band = nyf;
+    double best = 1e30;
+    for (int b = least; b < nyf && (best == 1e30 || b <= least + least / 4); ++b) {
+        if (walls && (nyf - 1) % b == 0) continue;
+        const int last = nyf % b ? nyf % b : b;
+        const double cost = 5.0 / last + 3.0 * (b - least) / least;
+        if (cost < best) { best = cost; band = b; }
+    }
     return std::max(1, band);
 }
 
