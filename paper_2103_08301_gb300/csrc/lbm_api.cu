@@ -352,26 +352,25 @@ int threads_of(const lbm_ctx *ctx)
 // strips). With walls no band boundary may fall between fluid rows 1|2 or
 // ny-3|ny-2 (fluid offsets 1 and nyf-1).
 //
-// A segment costs its rows and about five more for its halo, so the last band must
-// not be a few rows only: its CTAs would march through many short segments, and the
-// step waits for them. Higher bands than the share cost too (a CTA's rows then lie
-// in two strips, out of step with their neighbours: 14491 x 1739, share 268, a band
-// of 290 takes 443 us a step instead of 355), hence the weights below. FP32 row
-// pairs, us per step with the share itself and with the band chosen: 1999 x 1500,
-// last band of 4 rows, 58.6 and 51.1 (walls: 2 rows, 79.9 and 57.6); 5343 x 1244,
-// 3 rows, 143 and 98.6; 1180 x 741, 1 row, 37.4 and 21.2. 16384 x 2048 keeps its 359.
+// A segment costs its rows and about five more for its halo, so a last band of one
+// to five rows (and more than one strip) is avoided: its CTAs would march through
+// many short segments, and the step waits for them. The next height that leaves six
+// or none: no higher, since far above the share a CTA's rows lie in two strips, out
+// of step with their neighbours (14491 x 1739, share 268: 355 us a step; bands of 276
+// and 308, 376 and 462). FP32 row pairs, us per step with the share and with the band
+// chosen: 1999 x 1500, last band of 4 rows, 58.6 and 51.1 (walls: 2 rows, 79.9 and
+// 57.6); 5343 x 1244, 3 rows, 143 and 98.6; 1180 x 741, 1 row, 37.4 and 21.2. Six
+// rows or more do not show (4096 x 1024, 46 and 47: 10 and 35 rows, 73.1 and 72.9).
 int band_rows(int nyf, int nstrips, int nctas, int walls)
 {
     const long long share = ((long long)nyf * nstrips + nctas - 1) / nctas;
-    const int least = (int)std::min<long long>(nyf, std::max<long long>(8, share));
-    int band = nyf;
-    double best = 1e30;
-    for (int b = least; b < nyf && (best == 1e30 || b <= least + least / 4); ++b) {
-        if (walls && (nyf - 1) % b == 0) continue;
-        const int last = nyf % b ? nyf % b : b;
-        const double cost = 5.0 / last + 3.0 * (b - least) / least;
-        if (cost < best) { best = cost; band = b; }
-    }
+    int band = (int)std::min<long long>(nyf, std::max<long long>(8, share));
+    auto fits = [&](int b) { return !walls || b >= nyf || (nyf - 1) % b != 0; };
+    while (!fits(band)) ++band;
+    const int last = nyf % band;
+    if (nstrips > 1 && last > 0 && last < 6 && share >= std::max(6, 2 * last + 2))
+        for (int b = band + 1; b <= band + std::max(3, band / 4) && b < nyf; ++b)
+            if (fits(b) && (nyf % b == 0 || nyf % b >= 6)) { band = b; break; }
     return std::max(1, band);
 }
 
