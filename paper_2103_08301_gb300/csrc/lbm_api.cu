@@ -847,6 +847,25 @@ lbm_status plan_inplace_strips(lbm_ctx *ctx)
     return LBM_OK;
 }
 
+// Whether an FP32 step with solid nodes runs by row pairs (else the general-geometry
+// kernels, four to six of them: one more with walls, one with pressure columns). Row
+// pairs pay for the nodes that their strips of W columns are padded to, the others
+// for launches and for passes over memory. In us per step, row pairs against the
+// others. Neither walls nor pressure columns: 256 x 256, 11.4 and 10.6; 2048 x 256,
+// 25.1 and 22.1; 1024 x 1024, 37.3 and 38.4; 4096 x 1024, 95 and 153; narrow: 127 x
+// 5000, 38 and 26; 97 x 60000, 172 and 214. With either, narrow lattices of middle
+// size alone: 97 x 6000 (walls), 30.1 and 26.7; 250 x 3000, 34.2 and 32.1; 97 x 1000,
+// 13.3 and 14.9; 97 x 60000, 157 and 212; walls and columns, 130 x 4000, 31.5 and
+// 27.8; 130 x 30000, 133 and 149. Constants: nodes per SM.
+bool mask_pairs(const lbm_ctx *ctx)
+{
+    const double sms = ctx->sms, n = (double)ctx->grid.nx * ctx->grid.ny / sms,
+                 padded = (double)ctx->units * ctx->W / sms;
+    if (!ctx->grid.walls && !ctx->grid.bc_x) return n > 0.6 * padded + 2150;
+    const bool narrow = padded > 1.25 * n, short_runs = ctx->units / 2 <= 5 * ctx->sms;  // two rows a CTA
+    return !narrow || short_runs || n > 0.46 * padded + 1645;
+}
+
 // (Re)selects the general-geometry path: kept when the caller's mask adds
 // solid nodes to the wall rows or LBM_OPT_GENERAL forces it; the diagnostic
 // slots then follow its CTA count.
@@ -864,7 +883,7 @@ lbm_status plan_geometry(lbm_ctx *ctx)
                                     ctx->last_error, sizeof ctx->last_error);
     ctx->mask_rows2 = false;
     if (st != LBM_OK || !ctx->mask) return st;
-    if (ctx->rows2 && !ctx->big) {
+    if (ctx->rows2 && !ctx->big && mask_pairs(ctx)) {
         // the strip plan with this kernel's own residency
         ctx->tile = false;
         int per_sm = ctx->ctas_per_sm_opt;
