@@ -148,9 +148,10 @@ namespace lbm {
 // The FP64 step and fields by tiles (lbm_tile64.cu): tile height, grid and CTA
 // count for a lattice, and one launch over `ctas` CTAs (diagnostic slots).
 struct Tile64 {
-    int th, ntx, ntiles, sx, sy, ctas, threads;
+    int th, ntx, ntiles, sx, sy, ctas, threads, rot;
 };
 cudaError_t tile64_plan(int precision, int nx, int ny, bool walls, bool pres, bool big, int sms, Tile64 *p);
+void tile64_rotate(Tile64 *p, bool pres, int ctas);  // the order of the tiles for that many CTAs
 template <typename real>
 cudaError_t tile64_launch(const KArgs<real> &A, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
                           cudaStream_t st);

@@ -5,7 +5,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstdint>
+#include <vector>
 
 #include "lbm.h"
 #include "lbm_internal.h"
@@ -69,14 +71,36 @@ cudaError_t tile64_plan(int precision, int nx, int ny, bool walls, bool pres, bo
     if (e != cudaSuccess) return e;
     p->ctas = (int)std::min<long long>(ntiles, std::min<long long>(MAX_CTAS, (long long)sms * std::max(1, occ)));
     p->threads = T64_TX * p->th;
+    p->rot = 0;
     return cudaSuccess;
+}
+
+// Tile64::rot for a launch of `ctas`: of 0 .. 3 the one whose busiest CTA has the
+// fewest tiles with a pressure column, over up to 256 rows of tiles.
+void tile64_rotate(Tile64 *p, bool pres, int ctas)
+{
+    p->rot = 0;
+    if (!pres || p->ntiles <= ctas) return;
+    const int rows = std::min(p->ntiles / p->ntx, 256);
+    int least = INT_MAX;
+    std::vector<int> heavy(ctas);
+    for (int rot = 0; rot < std::min(p->ntx, 4); ++rot) {
+        std::fill(heavy.begin(), heavy.end(), 0);
+        int most = 0;
+        for (int by = 0; by < rows; ++by) {
+            const int turn = by * rot % p->ntx, first = turn ? p->ntx - turn : 0;  // where column 0 went
+            const int last = (first ? first : p->ntx) - 1;                          // and column ntx-1
+            for (const int r : {first, last}) most = std::max(most, ++heavy[(by * p->ntx + r) % ctas]);
+        }
+        if (most < least) { least = most; p->rot = rot; }
+    }
 }
 
 template <typename real>
 cudaError_t tile64_launch(const KArgs<real> &A, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
                           cudaStream_t st)
 {
-    T64Plan T{p.th, p.ntx, p.ntiles, p.sx, p.sy};
+    T64Plan T{p.th, p.ntx, p.ntiles, p.sx, p.sy, p.rot};
     void *args[] = {(void *)&A, (void *)&T};
     return cudaLaunchKernel(step_kernel_of<real>(walls, pres, big), dim3(ctas), dim3(p.threads), args, 0, st);
 }
@@ -160,7 +184,7 @@ cudaError_t fields_tiles(KArgs<real> A, const FieldsOut<real> &o, bool walls, bo
     Tile64 p;
     cudaError_t e = tile64_plan(sizeof(real) * 8, A.nx, A.ny, walls, pres, big, sms, &p);
     if (e != cudaSuccess) return e;
-    T64Plan T{p.th, p.ntx, p.ntiles, p.sx, p.sy};
+    T64Plan T{p.th, p.ntx, p.ntiles, p.sx, p.sy, 0};
     void *args[] = {(void *)&A, (void *)&T};
     // no per-CTA slots: enough CTAs for every SM's threads
     const int ctas = (int)std::min<long long>(p.ntiles, (long long)sms * 8);

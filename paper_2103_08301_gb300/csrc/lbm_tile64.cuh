@@ -52,12 +52,15 @@ struct SmemT64 {
 // would open a tile (its stencil is its neighbour's), one row down when no height
 // keeps the two rows next to a wall in one tile. CTAs stride over the tiles row of
 // tiles by row of tiles. A tile with a pressure column costs more (its lanes
-// extrapolate besides), and a stride that is a multiple of ntx (456 CTAs over 3, 4,
-// 6, 8, 12 columns of tiles) would give such tiles to the same CTAs always: each row
-// of tiles starts one tile further on (FP64, 97 x 60000: 3283 us a step without, 2611
-// with; 250 x 24000: 2619 and 1827; 4096 x 512: 563 and 551).
+// extrapolate besides), and where the stride comes back to the same column of tiles
+// within a few steps (456 CTAs over 3, 4, 6, 8, 12, 16 columns) the same CTAs would
+// get such tiles again and again: each row of tiles then starts rot tiles further on
+// than the one before, as the host finds best (tile64_rotate; FP64 us per step without
+// and with, 97 x 60000: 3283 and 2615; 250 x 24000: 2619 and 1832; 4096 x 512: 563 and
+// 552). A rotation that fits one width brings the columns back for another (2444 x
+// 941: 872 without, 986 with rot = 1).
 struct T64Plan {
-    int th, ntx, ntiles, sx, sy;
+    int th, ntx, ntiles, sx, sy, rot;
 };
 
 // row pointers of a shared array as the 3 x 3 operands of the stencils
@@ -97,10 +100,7 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
     for (int t = cta; t < T.ntiles; t += gridDim.x) {
         const int by = t / T.ntx;
         int bx = t - by * T.ntx;
-        if (PRES && T.ntiles > (int)gridDim.x) {  // see T64Plan
-            bx += by % T.ntx;
-            if (bx >= T.ntx) bx -= T.ntx;
-        }
+        if (PRES && T.rot) bx = (bx + by * T.rot) % T.ntx;
         const int x0 = bx * T64_TX - T.sx, y0 = yf0 + by * th - T.sy;
         const int xa = x0 + tx, r = y0 + ty;
         const bool active = xa >= 0 && xa < nx && r >= yf0 && r < yf1;
