@@ -765,11 +765,11 @@ struct CkptHeader {
 
 namespace {
 // A checkpoint's per-CTA partials for a plan of n CTAs: those of a plan with
-// more CTAs are folded into the first n, so that the totals stay.
+// more CTAs (m) are folded into the first n, so that the totals stay.
 template <typename real>
-void fold_partials(double *mass, double *J, real *ext, int n)
+void fold_partials(double *mass, double *J, real *ext, int n, int m)
 {
-    for (int c = n; c < lbm::MAX_CTAS; ++c) {
+    for (int c = n; c < m; ++c) {
         mass[c % n] += mass[c];
         J[c % n] += J[c];
         mass[c] = J[c] = 0.0;
@@ -1296,15 +1296,21 @@ lbm_status lbm_restore(lbm_ctx *ctx, const void *host_buf, size_t bytes)
     const int narr = ctx->inplace ? 1 : 2;
     const unsigned char *p = (const unsigned char *)host_buf + sizeof h;
     const size_t nparts = (size_t)lbm::MAX_CTAS * (16 + 4 * sz);
-    std::unique_ptr<unsigned char[]> part(new (std::nothrow) unsigned char[nparts]);
-    if (!part) return LBM_ERR_OOM;
+    const int own = diag_ctas(ctx), theirs = std::min<int>(h.nctas, lbm::MAX_CTAS);
+    std::unique_ptr<unsigned char[]> part;  // folded partials, where the file's plan had more CTAs
+    const unsigned char *mass = p + narr * ctx->L.pops;
+    if (theirs > own) {
+        part.reset(new (std::nothrow) unsigned char[nparts]);
+        if (!part) return LBM_ERR_OOM;
+        std::memcpy(part.get(), mass, nparts);
+        mass = part.get();
+        unsigned char *J = part.get() + lbm::MAX_CTAS * 8, *ext = J + lbm::MAX_CTAS * 8;
+        if (ctx->grid.precision == 64) fold_partials((double *)part.get(), (double *)J, (double *)ext, own, theirs);
+        else fold_partials((double *)part.get(), (double *)J, (float *)ext, own, theirs);
+    }
+    const unsigned char *J = mass + lbm::MAX_CTAS * 8, *ext = J + lbm::MAX_CTAS * 8;
     CK(cudaMemcpyAsync(ctx->ws + ctx->L.f0, p, narr * ctx->L.pops, cudaMemcpyHostToDevice, ctx->stream), "restore");
-    p += narr * ctx->L.pops;
-    std::memcpy(part.get(), p, nparts);
-    unsigned char *mass = part.get(), *J = mass + lbm::MAX_CTAS * 8, *ext = J + lbm::MAX_CTAS * 8;
-    if (ctx->grid.precision == 64) fold_partials((double *)mass, (double *)J, (double *)ext, diag_ctas(ctx));
-    else fold_partials((double *)mass, (double *)J, (float *)ext, diag_ctas(ctx));
-    p += nparts;
+    p += narr * ctx->L.pops + nparts;
     CK(cudaMemcpyAsync(ctx->ws + ctx->L.mass, mass, lbm::MAX_CTAS * 8, cudaMemcpyHostToDevice, ctx->stream), "restore");
     CK(cudaMemcpyAsync(ctx->ws + ctx->L.J, J, lbm::MAX_CTAS * 8, cudaMemcpyHostToDevice, ctx->stream), "restore");
     CK(cudaMemcpyAsync(ctx->ws + ctx->L.ext, ext, lbm::MAX_CTAS * 4 * sz, cudaMemcpyHostToDevice, ctx->stream), "restore");

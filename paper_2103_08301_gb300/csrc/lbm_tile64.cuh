@@ -57,8 +57,8 @@ struct SmemT64 {
 // get such tiles again and again: each row of tiles then starts rot tiles further on
 // than the one before, as the host finds best (tile64_rotate; FP64 us per step without
 // and with, 97 x 60000: 3283 and 2615; 250 x 24000: 2619 and 1832; 4096 x 512: 563 and
-// 552). A rotation that fits one width brings the columns back for another (2444 x
-// 941: 872 without, 986 with rot = 1).
+// 552). No one rotation fits all widths (2444 x 941: 986 with rot = 1, 621 with the
+// one chosen).
 struct T64Plan {
     int th, ntx, ntiles, sx, sy, rot;
 };
