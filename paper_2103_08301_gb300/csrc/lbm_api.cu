@@ -706,15 +706,19 @@ lbm_status do_fields(lbm_ctx *ctx, void *rho, void *ux, void *uy, void *tw, void
     lbm::KArgs<real> A = make_args<real>(ctx);
     if (ctx->mask) {
         A.fout = nullptr;
+        // solid nodes read zero: one pass over the scratch outputs, one over each
+        // direct one, none over those that nobody asked for
         real *p[5];
         size_t at = o.scratch;
+        if (o.scratch) CK(cudaMemsetAsync(ctx->fscratch, 0, o.scratch, ctx->stream), "fields memset");
         for (int k = 0; k < 5; ++k) {
             p[k] = o.ptr[k];
             if (!p[k]) {
                 p[k] = (real *)(ctx->fscratch + at);
                 at += align_up(o.bytes[k]);
+            } else if ((void *)p[k] == o.dst[k]) {
+                CK(cudaMemsetAsync(p[k], 0, o.bytes[k], ctx->stream), "fields memset");
             }
-            CK(cudaMemsetAsync(p[k], 0, o.bytes[k], ctx->stream), "fields memset");  // solid nodes
         }
         A.o_rho = p[0]; A.o_vx = p[1]; A.o_vy = p[2]; A.o_tw = p[3]; A.o_pw = p[4];
         CK(lbm::mask_launch<real>(ctx->mask, A, lbm::MODE_FIELDS, ctx->stream), "fields launch");
