@@ -458,7 +458,7 @@ lbm_status plan_launch(lbm_ctx *ctx)
         if (ctx->ctas_per_sm_opt > 0)
             ctx->nctas = (int)std::min<long long>({(long long)ctx->sms * ctx->ctas_per_sm_opt, ctx->t64p.ntiles,
                                                    lbm::MAX_CTAS});
-        lbm::tile64_rotate(&ctx->t64p, ctx->grid.bc_x, ctx->nctas);
+        lbm::tile64_rotate(&ctx->t64p, ctx->grid.bc_x && ctx->grid.precision == 64, ctx->nctas);
     }
     // short segments with tensor-load staging: one CTA per 32 x 8 tile instead
     // (no tile boundary between the wall-shear rows ny-3 | ny-2, and the
@@ -1596,7 +1596,7 @@ extern "C" lbm_status lbm_step_noalloc(const lbm_grid *grid, const lbm_eos *eos,
     if (plan_launch(&c) != LBM_OK) return LBM_ERR_CUDA;
     if (ctas > 0) c.nctas = (int)std::min<long long>(ctas, c.t64 ? c.t64p.ntiles : std::max<long long>(1, c.units / 2));
     c.nctas = std::min(c.nctas, NOALLOC_MAX_CTAS);
-    if (c.t64) lbm::tile64_rotate(&c.t64p, c.grid.bc_x, c.nctas);
+    if (c.t64) lbm::tile64_rotate(&c.t64p, c.grid.bc_x && c.grid.precision == 64, c.nctas);
     c.band = band_rows(c.nyf, c.nstrips, c.nctas, c.grid.walls);
     return grid->precision == 64 ? noalloc_launch<double>(&c, sc, f_in, f_out, diag_out, err_out)
                                  : noalloc_launch<float>(&c, sc, f_in, f_out, diag_out, err_out);

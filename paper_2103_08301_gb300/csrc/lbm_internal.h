@@ -151,7 +151,7 @@ struct Tile64 {
     int th, ntx, ntiles, sx, sy, ctas, threads, rot;
 };
 cudaError_t tile64_plan(int precision, int nx, int ny, bool walls, bool pres, bool big, int sms, Tile64 *p);
-void tile64_rotate(Tile64 *p, bool pres, int ctas);  // the order of the tiles for that many CTAs
+void tile64_rotate(Tile64 *p, bool on, int ctas);  // the order of the tiles for that many CTAs
 template <typename real>
 cudaError_t tile64_launch(const KArgs<real> &A, bool walls, bool pres, bool big, const Tile64 &p, int ctas,
                           cudaStream_t st);

@@ -43,7 +43,7 @@ void *step_kernel_of(bool walls, bool pres, bool big)
 // rows and about 1.2 more for its halo's densities, phi and Laplacians; at
 // 128 x 128 on 152 SMs that is 4, at 4096 x 512 it is 8). With walls the two rows
 // next to a wall share a tile (rows % th != 1). CTAs: a tile each up to the
-// slots of the per-CTA partials, then the resident CTAs stride over them.
+// resident ones (and the slots of the partials), which stride over the rest.
 cudaError_t tile64_plan(int precision, int nx, int ny, bool walls, bool pres, bool big, int sms, Tile64 *p)
 {
     void *fn = precision == 64 ? step_kernel_of<double>(walls, pres, big) : step_kernel_of<float>(walls, pres, false);
@@ -77,10 +77,10 @@ cudaError_t tile64_plan(int precision, int nx, int ny, bool walls, bool pres, bo
 
 // Tile64::rot for a launch of `ctas`: of 0 .. 3 the one whose busiest CTA has the
 // fewest tiles with a pressure column, over up to 256 rows of tiles.
-void tile64_rotate(Tile64 *p, bool pres, int ctas)
+void tile64_rotate(Tile64 *p, bool on, int ctas)
 {
     p->rot = 0;
-    if (!pres || p->ntiles <= ctas) return;
+    if (!on || p->ntiles <= ctas) return;
     const int rows = std::min(p->ntiles / p->ntx, 256);
     int least = INT_MAX;
     std::vector<int> heavy(ctas);

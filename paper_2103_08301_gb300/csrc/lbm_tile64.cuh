@@ -54,11 +54,12 @@ struct SmemT64 {
 // tiles by row of tiles. A tile with a pressure column costs more (its lanes
 // extrapolate besides), and where the stride comes back to the same column of tiles
 // within a few steps (456 CTAs over 3, 4, 6, 8, 12, 16 columns) the same CTAs would
-// get such tiles again and again: each row of tiles then starts rot tiles further on
-// than the one before, as the host finds best (tile64_rotate; FP64 us per step without
-// and with, 97 x 60000: 3283 and 2615; 250 x 24000: 2619 and 1832; 4096 x 512: 563 and
-// 552). No one rotation fits all widths (2444 x 941: 986 with rot = 1, 621 with the
-// one chosen).
+// get such tiles again and again: in FP64 each row of tiles then starts rot tiles
+// further on than the one before, as the host finds best (tile64_rotate; us per step
+// without and with, 97 x 60000: 3283 and 2615; 250 x 24000: 2619 and 1832; 4096 x 512:
+// 563 and 550). No one rotation fits all widths (2444 x 941: 986 with rot = 1, 620 with
+// the one chosen). In FP32 it brings nothing, and its code costs 1 to 3% (512 x 128: 5.28
+// and 5.45; 1024 x 256: 9.87 and 10.14).
 struct T64Plan {
     int th, ntx, ntiles, sx, sy, rot;
 };
@@ -100,7 +101,9 @@ __global__ void __launch_bounds__(T64_TX *T64_MAX, 3) step_kernel_tile64(const K
     for (int t = cta; t < T.ntiles; t += gridDim.x) {
         const int by = t / T.ntx;
         int bx = t - by * T.ntx;
-        if (PRES && T.rot) bx = (bx + by * T.rot) % T.ntx;
+        if constexpr (PRES && MODE == MODE_STEP && sizeof(real) == 8) {
+            if (T.rot) bx = (bx + by * T.rot) % T.ntx;
+        }
         const int x0 = bx * T64_TX - T.sx, y0 = yf0 + by * th - T.sy;
         const int xa = x0 + tx, r = y0 + ty;
         const bool active = xa >= 0 && xa < nx && r >= yf0 && r < yf1;
