@@ -179,10 +179,10 @@ lbm_status lbm_init(const lbm_grid *grid, const lbm_eos *eos, double tau, const 
  * otherwise. Even steps read each node's own slots and write its
  * post-collision populations back reversed; odd steps read from and write to
  * the neighbours' slots, restoring the natural layout. Each step runs two
- * kernels: the density of every fluid node into the plane (the stencil of
- * Eq. 2.17 reaches neighbours whose slots may already hold their next state),
- * then the collision from that plane; traffic is 116 bytes per node and step
- * (FP32) instead of 72. Populations are identical bit for bit to an lbm_init
+ * kernels: densities into the plane (the stencil of Eq. 2.17 reaches neighbours
+ * whose slots may already hold their next state), then the collision; traffic is
+ * 116 bytes per node and step (FP32) instead of 72, or about 74 on long FP32
+ * channels, which take from the plane only what lies outside a CTA's own rows. Populations are identical bit for bit to an lbm_init
  * context's; diagnostic sums agree to rounding (another summation order).
  * Arguments as lbm_init, without a wall mask (walls are the channel's rows 0
  * and ny-1 when grid->walls = 1); the workspace must hold
@@ -193,7 +193,7 @@ lbm_status lbm_init(const lbm_grid *grid, const lbm_eos *eos, double tau, const 
  * the one array and restore only into in-place contexts (LBM_ERR_STATE
  * otherwise); LBM_OPT_GENERAL and LBM_OPT_FAULT_SKIP_COPY are rejected
  * (LBM_ERR_ARG), and the kernel-selection options (LBM_OPT_STAGED, ROWS2,
- * TMA, TILE, STRIP, CTAS_PER_SM, PREFETCH, PDL) affect only lbm_fields.
+ * TMA, TILE, STRIP, CTAS_PER_SM, PREFETCH, PDL) have no effect.
  * lbm_launch_info reports the step's CTAs, its threads per CTA (FP32: 128,
  * two rows each; FP64: 256), its 32 x 8 tiles as units, and no staging; for
  * long FP32 channels, which step by row pairs in place, strip rows as units
@@ -295,9 +295,11 @@ lbm_status lbm_set_collision(lbm_ctx *ctx, const lbm_collision *c);
  *                        thread register prefetch. Both give identical results.
  *   LBM_OPT_ROWS2        nonzero (default): the staged FP32 step gives each
  *                        thread two rows of its column per iteration (paired
- *                        FP32 instructions) where it applies (staged, and nx a
- *                        multiple of 4 unless x has pressure columns); zero:
- *                        one row per iteration. Both give identical results.
+ *                        FP32 instructions) where it is the faster one (small
+ *                        grids step by tiles; a few narrow periodic widths that
+ *                        are not a multiple of 4, and some grids with solid
+ *                        nodes, a node per thread); zero: one row per
+ *                        iteration. All give identical populations.
  *   LBM_OPT_TMA          nonzero (default, contexts and batches):
  *                        the row-pair kernel stages each stencil row with one
  *                        2-D tensor (TMA) load; zero: nine bulk copies per
@@ -551,7 +553,11 @@ lbm_status lbm_plug_analysis(int32_t nx, int32_t ny, const double *rho, double r
  *   unless lbm_adjoint_set_precision says otherwise, on the stored states
  *   widened to FP64, so with 32 the result is the gradient of the FP64 step
  *   along the FP32 trajectory. nsteps >= 1.
- *   Allocates on the current device; stream as in lbm_init.
+ *   Allocates on the current device; stream as in lbm_init. Besides the states
+ *   above: 26 doubles a node, and two buffers for the fields of states that are
+ *   prepared while others are walked, 12 doubles a node and state, for as many
+ *   states as 256 MB hold (at least one, at most K) in either. Where these two
+ *   cannot be had, one state's 12 doubles a node (the same results, slower).
  * lbm_adjoint_forward: runs nsteps steps from f0 = f_eq(rho0, 0) under
  *   `drive` (NULL: no drive), keeping checkpoints, and returns J (host,
  *   2 doubles). rho0: nx*ny doubles, host or device. Synchronises the stream.

@@ -212,7 +212,9 @@ __device__ __forceinline__ void grad_term(T &gx, T &gy, int i, T v)
 // FP64 is bound by the number of FP64 instructions: its stencils add before
 // they scale. FP32 is not bound by arithmetic, and its sums over many nodes and
 // steps (J, dJ/d dp) show any change of rounding: its stencils add weighted
-// terms one by one in direction order, as every FP32 result so far was formed.
+// terms one by one in direction order. (adj_finish, which FP32 takes without
+// pressure columns or without walls, is written in the FP64 form for both; its FP32
+// gradients are as far from the FP64 sweep's as with the terms one by one.)
 template <typename T>
 constexpr bool BY_TERMS = sizeof(T) == 4;
 

@@ -443,7 +443,10 @@ lbm_status plan_launch(lbm_ctx *ctx)
                                              (int)dyn_smem(ctx));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "smem attribute");
     }
-    // Tiles (lbm_tile64.cuh): FP64 always (4096 x 512: 765 us by strips, 621 by tiles), FP32
+    // Tiles (lbm_tile64.cuh): FP64 always (us per step, strips against tiles, between
+    // pressure columns: 1024 x 256, 123 and 91; 4096 x 512, 628 and 552; 16384 x 2048, 9490
+    // and 8440; periodic: 1024 x 256, 95 and 83; 4096 x 512, 507 and 523, and from there
+    // on strips are 3 to 10% faster, which this rule leaves unused), FP32
     // up to 4096 nodes per SM, where a row-pair CTA marches so few rows that the
     // densities above and below its segment cost as much as its own (us per step, row
     // pairs against tiles: 512 x 128, 7.3 and 5.3; 1024 x 256, 12.6 and 10.0; 2048 x 256,
@@ -825,7 +828,8 @@ namespace {
 // are filled from the density plane, so short segments keep the tiles, whose cost
 // does not depend on segments (us per step, tiles against strips: 8192 x 1024,
 // 94 rows, 218 and 181; 8192 x 768, 70 rows, 166 and 141; 4096 x 1024, 47 rows,
-// 113 and 109; 4096 x 512, 24 rows, 53 and 65).
+// 113 and 109; 4096 x 512, 24 rows, 53 and 65). The two cross somewhere between 24
+// and 47 rows; the line is kept above both, at the cost of 4% just below it.
 constexpr long long AA_ROWS_MIN = 48;
 lbm_status plan_inplace_strips(lbm_ctx *ctx)
 {

@@ -18,13 +18,13 @@
 // The ghost sources are resolved on the host into a table of fluid (or
 // pressure-column) nodes per ghost point, so one gather per point fills them.
 //
-// FP32 steps (where the row-pair plan applies): two kernels. The ghost densities
+// FP32 steps (where mask_pairs of lbm_api.cu finds them faster): two kernels. The ghost densities
 // of the solid points within reach of the fluid are gathered, each from its few
 // sources' populations, and the row-pair kernel (lbm_rows2.cuh, MASK) does the
 // step with them, reading per point a 16-bit word of link and ghost flags: 74 B
 // per node and the rows around the obstacles instead of the 130 below. The 4096 x
 // 1024 channel with constrictions: 170 us a step in the six kernels below (which
-// remain for FP64, the fields and grids without row pairs), 107 us in these two.
+// remain for FP64, the fields and the other FP32 grids), 107 us in these two.
 //
 // Data (device, allocated by the library): the solid mask (1 B/node), three
 // ghost-extended arrays of (nx + 4)(ny + 4) values (density, phi, Laplacian),

@@ -33,8 +33,8 @@
 // Restricted to strips and pitches that are multiples of 4; a batch with
 // periodic x also to nx a multiple of 4 (its wrapped halo columns are copied as
 // one 16-byte group from each end of the row). A single channel's wrapped halo
-// lanes copy their own columns: a periodic width that is not a multiple of 4 ran
-// the one-row kernel before (1999 x 1501, Peng-Robinson, MRT: 71 us a step).
+// lanes copy their own columns, for any width (1999 x 1501, Peng-Robinson, MRT: 56 us
+// a step, 71 by the one-row kernel; that keeps a few narrow widths, plan_launch).
 #pragma once
 
 namespace lbm {
